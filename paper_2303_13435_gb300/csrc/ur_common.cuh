@@ -107,6 +107,43 @@ UR_HD __forceinline__ float2 twmul(float2 a, float2 w) {
 }
 
 // ---------------------------------------------------------------------------
+// Packed float32 pairs (add/mul/fma.f32x2): one instruction for two IEEE operations.  The
+// lanes per clock are those of the scalar forms (126 against 118 per SM measured), the
+// issue slots half as many, which is what the transforms are short of.
+// ---------------------------------------------------------------------------
+typedef unsigned long long ur_f2;
+__device__ __forceinline__ ur_f2 f2_pack(float a, float b) {
+  ur_f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2_get(ur_f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ ur_f2 f2_add(ur_f2 a, ur_f2 b) {
+  ur_f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ur_f2 f2_sub(ur_f2 a, ur_f2 b) {
+  ur_f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ur_f2 f2_mul(ur_f2 a, ur_f2 b) {
+  ur_f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ur_f2 f2_fma(ur_f2 a, ur_f2 b, ur_f2 c) {
+  ur_f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// ---------------------------------------------------------------------------
 // Small DFTs in registers.  Forward: y_p = sum_m a_m exp(-2 pi i m p / R);
 // inverse: the conjugate kernel (no scaling).
 // ---------------------------------------------------------------------------

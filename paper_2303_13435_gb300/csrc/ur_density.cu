@@ -13,45 +13,101 @@
 #include "ur_forward.cuh"
 #include "ur_density.cuh"
 
-template <typename T>
-__device__ __forceinline__ void store2(T* out, float a, float b);
-template <>
-__device__ __forceinline__ void store2<float>(float* out, float a, float b) {
-  *reinterpret_cast<float2*>(out) = make_float2(a, b);
-}
-template <>
-__device__ __forceinline__ void store2<__half>(__half* out, float a, float b) {
-  *reinterpret_cast<__half2*>(out) = __halves2half2(__float2half_rn(a), __float2half_rn(b));
+// W neighbouring voxels of a row (W = 2, or 8 where every row starts on a 16-byte boundary)
+template <typename T, int W>
+__device__ __forceinline__ void store_row(T* out, const float (&v)[W]) {
+  if constexpr (W == 2 && sizeof(T) == 4) {
+    *reinterpret_cast<float2*>(out) = make_float2(v[0], v[1]);
+  } else if constexpr (W == 2) {
+    *reinterpret_cast<__half2*>(out) = __halves2half2(__float2half_rn(v[0]), __float2half_rn(v[1]));
+  } else if constexpr (sizeof(T) == 4) {
+    reinterpret_cast<float4*>(out)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(out)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
+    __half2 h[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = __halves2half2(__float2half_rn(v[2 * i]), __float2half_rn(v[2 * i + 1]));
+    *reinterpret_cast<uint4*>(out) = *reinterpret_cast<const uint4*>(h);
+  }
 }
 
-// grid (ceil(N*N/2 / blockDim), z_count): each thread writes two neighbouring voxels of a row
-template <typename T, bool LAT>
-__global__ void __launch_bounds__(256) k_density(int N, const float* __restrict__ cell, int U, int ox, int oy, int oz,
-                                                 ShapeArgs sh, LatArgs lat, const float* __restrict__ weights,
-                                                 int z_begin, T* __restrict__ out, int* __restrict__ nz_range) {
-  const int z = z_begin + blockIdx.y;
-  const long long pair = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long plane_pairs = (long long)N * N / 2;
+struct DensityArgs {
+  int N, U, ox, oy, z_begin, z_org;  // cell plane of plane blockIdx.y: (z_org + blockIdx.y) mod U
+  const float* cell;
+  int vec;        // 1: every group of 4 voxels is one aligned 16-byte read of the cell row
+  int lg_lanes;   // threads per row: 2^lg_lanes
+  FastDiv fu;     // division by U
+  ShapeArgs sh;
+  LatArgs lat;
+  const float* weights;
+};
+
+// Grid (rows of a plane / rows per block, z_count); 2^lg_lanes neighbouring threads write a row in
+// groups of W voxels.  Bound by the writes of the density, so what a row shares (cell row, the y and
+// z terms of the mask) is formed once per thread and a group's mask costs two voxels, not W, where
+// the float32 predicate is an interval along the row (RowMask::group); the values are always u * m.
+// 1024^3 FP16 cube filling the box: 4294 -> 615 us (two voxels per thread with 64-bit divisions,
+// every voxel's mask evaluated; one group per thread, 938 us).
+template <typename T, bool LAT, int W>
+__global__ void __launch_bounds__(256) k_density(const __grid_constant__ DensityArgs a, T* __restrict__ out,
+                                                 int* __restrict__ nz_range) {
+  const int N = a.N, U = a.U;
+  const int z = a.z_begin + blockIdx.y;
+  const int lanes = 1 << a.lg_lanes;
+  const int y = (int)(blockIdx.x * (256u >> a.lg_lanes) + (threadIdx.x >> a.lg_lanes));
   bool nonzero = false;
-  if (pair < plane_pairs) {
-    const int y = (int)(pair / (N / 2));
-    const int x = (int)(pair - (long long)y * (N / 2)) * 2;
-    const int cz = (z + oz) % U, cy = (y + oy) % U;
-    const float* crow = cell + ((long long)cz * U + cy) * U;
-    float v[2];
+  if (y < N) {
+    const float* crow = a.cell + ((long long)a.fu.mod((uint32_t)(a.z_org + (int)blockIdx.y)) * U +
+                                  a.fu.mod((uint32_t)(y + a.oy))) * U;
+    const int x0 = (threadIdx.x & (lanes - 1)) * W;
+    int c = (int)a.fu.mod((uint32_t)(x0 + a.ox));
+    const int cstep = (int)a.fu.mod((uint32_t)(lanes * W));
+    RowMask rm;
+    rm.init(a.sh, y, z);
+    T* orow = out + ((long long)blockIdx.y * N + y) * N;
+    for (int x = x0; x < N; x += lanes * W) {
+      float u[W], m[W], v[W];
+      if (LAT) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int xx = x + e;
-      const float u = LAT ? lattice_sample(lat, sh, cell, U, xx, y, z) : __ldg(crow + (xx + ox) % U);
-      float m;
-      if (sh.kind == UR_SHAPE_WEIGHTS) m = __ldg(weights + ((long long)z * N + y) * N + xx);
-      else m = mask_at(sh, xx, y, z);
-      v[e] = __fmul_rn(u, m);
-      // nonzero as stored (an FP16 value may round to zero)
-      if (sizeof(T) == 2) v[e] = __half2float(__float2half_rn(v[e]));
+        for (int e = 0; e < W; ++e) u[e] = lattice_sample(a.lat, a.sh, a.cell, U, x + e, y, z);
+      } else {
+        int ce = c;
+        if (W == 8 && a.vec) {
+#pragma unroll
+          for (int h = 0; h < W / 4; ++h) {
+            const float4 t = __ldg(reinterpret_cast<const float4*>(crow + ce));
+            u[4 * h] = t.x;
+            u[4 * h + 1] = t.y;
+            u[4 * h + 2] = t.z;
+            u[4 * h + 3] = t.w;
+            ce = ce + 4 == U ? 0 : ce + 4;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < W; ++e) {
+            u[e] = __ldg(crow + ce);
+            ce = ce + 1 == U ? 0 : ce + 1;
+          }
+        }
+        c += cstep;
+        if (c >= U) c -= U;
+      }
+      if (a.sh.kind == UR_SHAPE_WEIGHTS) {
+        const float* wrow = a.weights + ((long long)z * N + y) * N + x;
+#pragma unroll
+        for (int e = 0; e < W; ++e) m[e] = __ldg(wrow + e);
+      } else {
+        rm.group<W>(x, m);
+      }
+#pragma unroll
+      for (int e = 0; e < W; ++e) v[e] = __fmul_rn(u[e], m[e]);
+      if (nz_range) {
+        // nonzero as stored (an FP16 value may round to zero)
+#pragma unroll
+        for (int e = 0; e < W; ++e) nonzero |= (sizeof(T) == 2 ? __half2float(__float2half_rn(v[e])) : v[e]) != 0.f;
+      }
+      store_row<T, W>(orow + x, v);
     }
-    nonzero = (v[0] != 0.f) || (v[1] != 0.f);
-    store2<T>(out + ((long long)blockIdx.y * N + y) * N + x, v[0], v[1]);
   }
   if (nz_range) {
     if (__syncthreads_or(nonzero) && threadIdx.x == 0) {
@@ -91,21 +147,41 @@ static ur_status build_density(int32_t n, const float* cell, int32_t ucell, cons
   const LatArgs lat = ur_lattice_args(lattice);
   if (z_count == 0) return UR_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  const long long pairs = (long long)n * n / 2;
-  dim3 grid((unsigned)((pairs + 255) / 256), (unsigned)z_count);
+  DensityArgs a;
+  memset(&a, 0, sizeof a);
+  a.N = n;
+  a.U = ucell;
+  // cell indices by multiply-shift need x + origin < 2^31: the origin reduced modulo the cell edge
+  a.ox = ox % ucell;
+  a.oy = oy % ucell;
+  a.z_begin = z_begin;
+  a.z_org = oz % ucell + z_begin;
+  a.cell = cell;
+  a.fu = FastDiv((uint32_t)ucell);
+  a.sh = sh;
+  a.lat = lat;
+  a.weights = weights;
+  // groups of eight voxels need 16-byte row starts; edges that are no multiple of 8 (and the
+  // rotated lattice, bound by its eight cell reads per voxel) take pairs
+  const bool wide = n % 8 == 0 && ((uintptr_t)ed_out % 16) == 0 && !lat.on;
+  a.vec = (ucell % 4 == 0 && a.ox % 4 == 0 && ((uintptr_t)cell % 16) == 0) ? 1 : 0;
+  // a warp per row, or as many threads (a power of two) as a short row has groups
+  const int per_row = n / (wide ? 8 : 2);
+  while (a.lg_lanes < 5 && (1 << a.lg_lanes) < per_row) ++a.lg_lanes;
+  const int rows = 256 >> a.lg_lanes;
+  dim3 grid((unsigned)((n + rows - 1) / rows), (unsigned)z_count);
   ur_timing_begin("density", s);
-  if (out_dtype == UR_F32 && !lat.on)
-    k_density<float, false><<<grid, 256, 0, s>>>(n, cell, ucell, ox, oy, oz, sh, lat, weights, z_begin, (float*)ed_out,
-                                                 nz_range);
-  else if (out_dtype == UR_F32)
-    k_density<float, true><<<grid, 256, 0, s>>>(n, cell, ucell, ox, oy, oz, sh, lat, weights, z_begin, (float*)ed_out,
-                                                nz_range);
-  else if (!lat.on)
-    k_density<__half, false><<<grid, 256, 0, s>>>(n, cell, ucell, ox, oy, oz, sh, lat, weights, z_begin,
-                                                  (__half*)ed_out, nz_range);
-  else
-    k_density<__half, true><<<grid, 256, 0, s>>>(n, cell, ucell, ox, oy, oz, sh, lat, weights, z_begin,
-                                                 (__half*)ed_out, nz_range);
+  int* nzr = nz_range;
+  if (wide) {
+    if (out_dtype == UR_F32) k_density<float, false, 8><<<grid, 256, 0, s>>>(a, (float*)ed_out, nzr);
+    else k_density<__half, false, 8><<<grid, 256, 0, s>>>(a, (__half*)ed_out, nzr);
+  } else if (!lat.on) {
+    if (out_dtype == UR_F32) k_density<float, false, 2><<<grid, 256, 0, s>>>(a, (float*)ed_out, nzr);
+    else k_density<__half, false, 2><<<grid, 256, 0, s>>>(a, (__half*)ed_out, nzr);
+  } else {
+    if (out_dtype == UR_F32) k_density<float, true, 2><<<grid, 256, 0, s>>>(a, (float*)ed_out, nzr);
+    else k_density<__half, true, 2><<<grid, 256, 0, s>>>(a, (__half*)ed_out, nzr);
+  }
   UR_LAUNCH_CHECK("k_density");
   ur_timing_end(s);
   return UR_OK;
@@ -156,6 +232,140 @@ __device__ __forceinline__ unsigned short half_bits_from_fixed24(long long S) {
   const int ex = e - 9;  // biased exponent of q * 2^(e - 10 - 24)
   if (ex >= 31) return sign | 0x7C00;
   return sign | (unsigned short)((ex << 10) | (int)(q - 1024ull));
+}
+
+// FP16 block sums for f = 2, 4, 8, 16 and rows of whole 16-byte groups.  One block per output row
+// (Z, Y) of the particle, then blocks that zero the other rows; a thread sums the f^2 source rows of 8 neighbouring x.  Bound by the reads of the
+// source, so the exact integer sum must be cheap: with C = 1.5 2^17 every t = v + C lies in
+// [2^17, 2^18), where floats are multiples of 2^-6, so the bits of t count v rounded to 2^-6
+// (summed as int32) and v - (t - C), a multiple of 2^-24 of at most 2^-7, is summed exactly in
+// float32 over up to 128 terms before it is added to an integer.  A source row with an infinity or
+// NaN shows as a NaN remainder; its outputs take the conversion of k_zoom.
+// 1024^3 -> 512^3 box by 4 / by 16: 1847 / 1918 -> 461 / 395 us (two-byte loads, a
+// 64-bit conversion per value, 64-bit shared atomics).
+#define UR_ZOOM_C 196608.0f
+#define UR_ZOOM_ZROWS 16  // rows of the box per zero-filling block
+template <int F, typename TO>
+__global__ void __launch_bounds__(256) k_zoom_half(const __half* __restrict__ src, int n_src, int n_out,
+                                                   TO* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  long long* acc = reinterpret_cast<long long*>(smraw);
+  const int m = n_src / F, o = (n_out - m) / 2;
+  const bool wide = n_out % 8 == 0 && ((uintptr_t)out % 16) == 0;  // rows start on 16-byte boundaries
+  if (blockIdx.x >= (unsigned)(m * m)) {  // rows that no source row reaches
+    const long long r0 = (long long)(blockIdx.x - m * m) * UR_ZOOM_ZROWS;
+    for (long long r = r0; r < r0 + UR_ZOOM_ZROWS && r < (long long)n_out * n_out; ++r) {
+      const int Zr = (int)(r / n_out) - o, Yr = (int)(r % n_out) - o;
+      if (Zr >= 0 && Zr < m && Yr >= 0 && Yr < m) continue;
+      TO* row = out + r * n_out;
+      if (wide) {
+        for (int X = threadIdx.x; X < n_out * (int)sizeof(TO) / 16; X += blockDim.x)
+          reinterpret_cast<uint4*>(row)[X] = make_uint4(0u, 0u, 0u, 0u);
+      } else {
+        for (int X = threadIdx.x; X < n_out; X += blockDim.x) row[X] = TO(0.f);
+      }
+    }
+    return;
+  }
+  const int zs = blockIdx.x / m, ys = blockIdx.x - (blockIdx.x / m) * m;
+  TO* orow = out + ((long long)(zs + o) * n_out + (ys + o)) * n_out;
+  constexpr int PER = 8 / F > 0 ? 8 / F : 1;   // outputs per thread (F = 16: two threads share one)
+  constexpr int NV = F < 8 ? F : 8;            // values of a thread's row group per output
+  constexpr int FOLD = 128 < F * F ? 128 / F : F;  // dz per fold: at most 128 terms per float32 sum
+  {
+    const int groups = n_src / 8;
+    const int rounds = (groups + (int)blockDim.x - 1) / (int)blockDim.x;
+    for (int it = 0; it < rounds; ++it) {
+      const int g = threadIdx.x + it * blockDim.x;
+      long long S[PER];
+#pragma unroll
+      for (int p = 0; p < PER; ++p) S[p] = 0;
+      if (g < groups) {
+        const __half* base = src + ((long long)F * zs * n_src + (long long)F * ys) * n_src + 8 * g;
+        int hi[8], lo[8];
+        bool bad = false;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) hi[e] = lo[e] = 0;
+        const ur_f2 C = f2_pack(UR_ZOOM_C, UR_ZOOM_C);
+        for (int z0 = 0; z0 < F; z0 += FOLD) {
+          ur_f2 rem[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) rem[q] = f2_pack(0.f, 0.f);
+#pragma unroll(F <= 4 ? FOLD : 1)
+          for (int dz = z0; dz < z0 + FOLD; ++dz) {
+#pragma unroll
+            for (int dy = 0; dy < F; ++dy) {
+              const uint4 w = __ldg(reinterpret_cast<const uint4*>(base + ((long long)dz * n_src + dy) * n_src));
+              const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ww[q]));
+                const ur_f2 v = f2_pack(f.x, f.y);
+                const ur_f2 t = f2_add(v, C);
+                rem[q] = f2_add(rem[q], f2_sub(v, f2_sub(t, C)));
+                const float2 tt = f2_get(t);
+                hi[2 * q] += __float_as_int(tt.x) - __float_as_int(UR_ZOOM_C);
+                hi[2 * q + 1] += __float_as_int(tt.y) - __float_as_int(UR_ZOOM_C);
+              }
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float2 r = f2_get(rem[q]);
+            bad |= r.x != r.x || r.y != r.y;
+            lo[2 * q] += __float2int_rn(r.x * 16777216.0f);
+            lo[2 * q + 1] += __float2int_rn(r.y * 16777216.0f);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) S[e / NV] += ((long long)hi[e] << 18) + (long long)lo[e];
+        if (bad) {
+#pragma unroll
+          for (int p = 0; p < PER; ++p) S[p] = 0;
+          for (int dz = 0; dz < F; ++dz)
+            for (int dy = 0; dy < F; ++dy)
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                S[e / NV] += __float2ll_rn(__half2float(base[((long long)dz * n_src + dy) * n_src + e]) * 16777216.0f);
+        }
+      }
+      if constexpr (F == 16) S[0] += __shfl_xor_sync(0xffffffffu, S[0], 1);  // rounds are uniform over the block
+      if (g < groups) {
+        if constexpr (F == 16) {
+          if ((g & 1) == 0) acc[g / 2] = S[0];
+        } else {
+#pragma unroll
+          for (int p = 0; p < PER; ++p) acc[g * PER + p] = S[p];
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // eight outputs per thread where rows start on 16-byte boundaries, else one
+  const int step = wide ? 8 : 1;
+  for (int X = threadIdx.x * step; X < n_out; X += blockDim.x * step) {
+    float vf[8];
+    unsigned short hb[8];
+    for (int e = 0; e < step; ++e) {
+      const int xs = X + e - o;
+      const long long S = (xs >= 0 && xs < m) ? acc[xs] : 0;
+      if constexpr (sizeof(TO) == 2) hb[e] = half_bits_from_fixed24(S);
+      else vf[e] = __double2float_rn((double)S * 5.9604644775390625e-08);  // * 2^-24, exact in double
+    }
+    if (wide) {
+      if constexpr (sizeof(TO) == 2) {
+        *reinterpret_cast<uint4*>(orow + X) =
+            make_uint4(hb[0] | (uint32_t)hb[1] << 16, hb[2] | (uint32_t)hb[3] << 16, hb[4] | (uint32_t)hb[5] << 16,
+                       hb[6] | (uint32_t)hb[7] << 16);
+      } else {
+        reinterpret_cast<float4*>(orow + X)[0] = make_float4(vf[0], vf[1], vf[2], vf[3]);
+        reinterpret_cast<float4*>(orow + X)[1] = make_float4(vf[4], vf[5], vf[6], vf[7]);
+      }
+    } else {
+      if constexpr (sizeof(TO) == 2) orow[X] = __ushort_as_half(hb[0]);
+      else orow[X] = vf[0];
+    }
+  }
 }
 
 // One block per output row (Z, Y) of the n_out^3 box.
@@ -231,11 +441,31 @@ extern "C" ur_status ur_zoom_density(int32_t n_src, int32_t src_dtype, const voi
     k_zoom<TS, TO><<<grid, 256, smem, s>>>((const TS*)src, n_src, f, n_out, (TO*)out);                    \
   } while (0)
   ur_timing_begin("zoom", s);
-  if (src_dtype == UR_F16 && out_dtype == UR_F16) UR_ZOOM(__half, __half);
+  // FP16 sources with the usual factors and rows of whole 16-byte groups: k_zoom_half; every other
+  // factor, edge, alignment and FP32 sources: k_zoom
+  const bool fast = src_dtype == UR_F16 && n_src % 8 == 0 && ((uintptr_t)src % 16) == 0;
+#define UR_ZOOM_HALF(F)                                                                                   \
+  do {                                                                                                    \
+    const int threads = n_src / 8 >= 256 ? 256 : (n_src / 8 + 31) / 32 * 32;                              \
+    if (smem > 48 * 1024) {                                                                               \
+      UR_CUDA_CHECK(cudaFuncSetAttribute(k_zoom_half<F, __half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+      UR_CUDA_CHECK(cudaFuncSetAttribute(k_zoom_half<F, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  \
+    }                                                                                                     \
+    const unsigned zgrid = (unsigned)((long long)m * m + ((long long)n_out * n_out + UR_ZOOM_ZROWS - 1) / UR_ZOOM_ZROWS); \
+    if (out_dtype == UR_F16)                                                                              \
+      k_zoom_half<F, __half><<<zgrid, threads, smem, s>>>((const __half*)src, n_src, n_out, (__half*)out); \
+    else k_zoom_half<F, float><<<zgrid, threads, smem, s>>>((const __half*)src, n_src, n_out, (float*)out); \
+  } while (0)
+  if (fast && f == 2) UR_ZOOM_HALF(2);
+  else if (fast && f == 4) UR_ZOOM_HALF(4);
+  else if (fast && f == 8) UR_ZOOM_HALF(8);
+  else if (fast && f == 16) UR_ZOOM_HALF(16);
+  else if (src_dtype == UR_F16 && out_dtype == UR_F16) UR_ZOOM(__half, __half);
   else if (src_dtype == UR_F16) UR_ZOOM(__half, float);
   else if (out_dtype == UR_F16) UR_ZOOM(float, __half);
   else UR_ZOOM(float, float);
 #undef UR_ZOOM
+#undef UR_ZOOM_HALF
   UR_LAUNCH_CHECK("k_zoom");
   ur_timing_end(s);
   return UR_OK;

@@ -62,6 +62,49 @@ struct RowMask {
   __device__ __forceinline__ bool empty() const {
     return kind == UR_SHAPE_SPHERE && __fadd_rn(dy2, dz2) > s2;
   }
+  // Signed coordinate of axis a at x, rounded as in mask_at; nondecreasing or nonincreasing in x,
+  // since rounding to nearest is monotone
+  __device__ __forceinline__ float coord(int a, float dx) const {
+    return __fadd_rn(__fadd_rn(__fmul_rn(r0[a], dx), ry[a]), rz[a]);
+  }
+  // Mask values of the W voxels from x on.  Sphere and cube predicates hold on an interval of the
+  // row (each side of the sphere's centre and each cube coordinate is monotone in x, roundings
+  // included), so a group whose end voxels are both inside is inside, and one whose end voxels fail
+  // the same side of the predicate is outside; other groups, and the octahedron (a rounded sum of
+  // three coordinates, not an interval), take every voxel.
+  template <int W>
+  __device__ __forceinline__ void group(int x, float (&m)[W]) const {
+    if constexpr (W > 2) {
+      if (kind == UR_SHAPE_ALL) {
+#pragma unroll
+        for (int e = 0; e < W; ++e) m[e] = 1.f;
+        return;
+      }
+      bool in = false, out = false;
+      const float da = __fsub_rn((float)x, cx), db = __fsub_rn((float)(x + W - 1), cx);
+      if (kind == UR_SHAPE_SPHERE) {
+        const bool ia = __fadd_rn(__fadd_rn(__fmul_rn(da, da), dy2), dz2) <= s2;
+        const bool ib = __fadd_rn(__fadd_rn(__fmul_rn(db, db), dy2), dz2) <= s2;
+        in = ia && ib;
+        out = !ia && !ib && (da >= 0.f || db <= 0.f);
+      } else if (kind == UR_SHAPE_CUBE) {
+        in = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const float ta = coord(a, da), tb = coord(a, db);
+          in = in && fabsf(ta) <= s && fabsf(tb) <= s;
+          out = out || (ta > s && tb > s) || (ta < -s && tb < -s);
+        }
+      }
+      if (in || out) {
+#pragma unroll
+        for (int e = 0; e < W; ++e) m[e] = in ? 1.f : 0.f;
+        return;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < W; ++e) m[e] = at(x + e);
+  }
   __device__ __forceinline__ float at(int x) const {
     if (kind == UR_SHAPE_ALL) return 1.f;
     const float dx = __fsub_rn((float)x, cx);
