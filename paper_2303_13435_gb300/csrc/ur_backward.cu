@@ -77,7 +77,7 @@ __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int
         const int a = (int)dNy.div((uint32_t)q);
         const int b = q - a * nyr;
         const long long z = zf + (long long)U * a, y = yf + (long long)U * b;
-        const float2* row = Y + (z * N + y) * H;
+        const float2* row = Y + (z * N + y) * g.yp;
         const float2 xa = __ldg(row + i), xb = __ldg(row + (M - i));
         const float2 w = __ldg(tw + i);
         const float2 e = cadd(xa, cconj(xb));
@@ -96,7 +96,7 @@ __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int
           const int a = (int)dNy.div((uint32_t)q);
           const int b = q - a * nyr;
           const long long z = zf + (long long)U * a, y = yf + (long long)U * b;
-          v = __ldg(Y + (z * N + y) * H + k);
+          v = __ldg(Y + (z * N + y) * g.yp + k);
         }
         buf[f] = v;
       }
@@ -260,14 +260,16 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   // B1
   ColArgs a = ur_col_args(p);
   a.ncols = (long long)n * H;
-  a.A = H;
-  a.S = (long long)n * H;
-  a.Ad = H;
-  a.Sd = (long long)n * H;
+  a.A = p->xp;
+  a.S = (long long)n * p->xp;
+  a.Ad = p->xp;
+  a.Sd = (long long)n * p->xp;
   a.dst = Y;
   a.sigma = sigma;
-  if (F) {
+  if (F) {  // caller's layout: rows of N/2+1
     a.src = (const float2*)F;
+    a.A = H;
+    a.S = (long long)n * H;
     a.nload = n;
     a.zoff = 0;
     a.skip_fwd = 1;
@@ -317,11 +319,11 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
     for (int p0 = 0; p0 < n; p0 += p->chunk_planes) {
       const int np = (p0 + p->chunk_planes <= n) ? p->chunk_planes : n - p0;
       ColArgs b = ur_col_args(p);
-      b.src = Y + (long long)p0 * n * H;
+      b.src = Y + (long long)p0 * n * p->xp;
       b.dst = whole ? Y : C;
       b.ncols = (long long)np * H;
-      b.A = (long long)n * H;
-      b.S = H;
+      b.A = (long long)n * p->xp;
+      b.S = p->xp;
       b.Ad = b.A;
       b.Sd = b.S;
       b.nload = n;
@@ -332,6 +334,7 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
       UR_TRY(ur_fast_cols(n, 1 /* y inverse */, b, s));
       ur_timing_end(s);
       g.Y = whole ? Y : C;
+      g.yp = p->xp;
       g.ybase_z = p0;
       g.z0 = p0;
       ur_timing_begin("adj_rows_grad", s);
@@ -346,8 +349,8 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   b.src = Y;
   b.dst = Y;
   b.ncols = (long long)n * H;
-  b.A = (long long)n * H;
-  b.S = H;
+  b.A = (long long)n * p->xp;
+  b.S = p->xp;
   b.Ad = b.A;
   b.Sd = b.S;
   b.nload = n;
@@ -377,6 +380,7 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   GenGradArgs ga;
   memset(&ga, 0, sizeof ga);
   ga.Y = Y;
+  ga.yp = p->xp;
   ga.N = n;
   ga.RB = RB;
   ga.nst = p->sched_m.nst;
@@ -490,7 +494,7 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
   float2* X = (float2*)ws;
   char* o = (char*)ws + ur_align_up(p->ws_inter, 256) + 2 * ur_align_up(p->ws_slab, 256);
   float2* Ys = (float2*)o;
-  o += ur_align_up((size_t)S * n * H * sizeof(float2), 256);
+  o += ur_align_up((size_t)S * n * p->xp * sizeof(float2), 256);
   float* sigma = (float*)o;
   o += ur_align_up(p->ws_sigma, 256);
   float* dm[2];
@@ -538,10 +542,10 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
     // z pass over every column, keeping planes [za, za + cnt)
     ColArgs a = ur_col_args(p);
     a.ncols = (long long)n * H;
-    a.A = H;
-    a.S = (long long)n * H;
-    a.Ad = H;
-    a.Sd = (long long)n * H;
+    a.A = p->xp;
+    a.S = (long long)n * p->xp;
+    a.Ad = p->xp;
+    a.Sd = (long long)n * p->xp;
     a.src = X;
     a.nload = p->nz;
     a.zoff = p->z0;
@@ -559,8 +563,8 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
     c.src = Ys;
     c.dst = Ys;
     c.ncols = (long long)cnt * H;
-    c.A = (long long)n * H;
-    c.S = H;
+    c.A = (long long)n * p->xp;
+    c.S = p->xp;
     c.Ad = c.A;
     c.Sd = c.S;
     c.nload = n;
@@ -577,6 +581,7 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
       const int b = sub & 1;
       if (dl_dmask_host && sub >= 2) cudaStreamWaitEvent(s, freed[b], 0);
       g.Y = Ys;
+      g.yp = p->xp;
       g.ybase_z = za;
       g.z0 = zb;
       g.dl_dmask = dl_dmask_host ? dm[b] : nullptr;

@@ -117,6 +117,7 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     BatchRowsItem& r = rows[i];
     memset(&r, 0, sizeof r);
     r.ra.X = X;
+    r.ra.xp = p->xp;
     r.ra.nrows = (long long)p->nz * n;
     r.ra.z0 = p->z0;
     r.ra.cell = it.cell;
@@ -139,8 +140,8 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     a.src = X;
     a.dst = X;
     a.ncols = (long long)p->nz * H;
-    a.A = (long long)n * H;
-    a.S = H;
+    a.A = (long long)n * p->xp;
+    a.S = p->xp;
     a.Ad = a.A;
     a.Sd = a.S;
     a.nload = n;
@@ -153,8 +154,8 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     ColArgs zb_ = ur_col_args(p);
     zb_.src = X;
     zb_.ncols = (long long)n * H;
-    zb_.A = H;
-    zb_.S = (long long)n * H;
+    zb_.A = p->xp;
+    zb_.S = (long long)n * p->xp;
     zb_.nload = p->nz;
     zb_.zoff = p->z0;
     zb_.iscale = (float)(1.0 / n3);
@@ -179,10 +180,10 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     za.src = X;
     za.dst = Y;
     za.ncols = (long long)n * H;
-    za.A = H;
-    za.S = (long long)n * H;
-    za.Ad = H;
-    za.Sd = (long long)n * H;
+    za.A = p->xp;
+    za.S = (long long)n * p->xp;
+    za.Ad = p->xp;
+    za.Sd = (long long)n * p->xp;
     za.nload = p->nz;
     za.zoff = p->z0;
     za.sigma = sigma;
@@ -192,8 +193,8 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     yi.src = Y;
     yi.dst = Y;
     yi.ncols = (long long)n * H;
-    yi.A = (long long)n * H;
-    yi.S = H;
+    yi.A = (long long)n * p->xp;
+    yi.S = p->xp;
     yi.Ad = yi.A;
     yi.Sd = yi.S;
     yi.nload = n;
@@ -206,6 +207,7 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     BatchGradItem& g = grad[i];
     memset(&g, 0, sizeof g);
     g.g.Y = Y;
+    g.g.yp = p->xp;
     g.g.N = n;
     g.g.RB = p->row_rb;
     g.g.nst = p->sched_m.nst;

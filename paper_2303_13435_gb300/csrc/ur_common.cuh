@@ -708,6 +708,7 @@ __device__ __forceinline__ void ur_finalize_shifted(double* __restrict__ bins, c
 // ---------------------------------------------------------------------------
 struct ur_plan {
   int n, M, H;       // grid edge, N/2, N/2+1
+  int xp;            // row pitch of the intermediates X and Y, complex values (N/2+1, or that rounded up to 32 bytes)
   double dx, dq;
   int ed_dtype, z0, nz, nbins;
   int device, num_sms;

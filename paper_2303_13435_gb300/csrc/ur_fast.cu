@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
     // Z[M - k], k = j + qT, is register 7 - q of lane T - j of the same row (j >= 1);
     // lane j = 0 holds its own partners: Z[M - qT] = its register 8 - q, and Z[0]
     const int src = ((threadIdx.x & 31) & ~(T - 1)) | ((T - j) & (T - 1));
-    float2* X = a.X + (valid ? r : 0) * H;
+    float2* X = a.X + (valid ? r : 0) * a.xp;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       float2 zm = make_float2(__shfl_sync(wmask, v[7 - q].x, src), __shfl_sync(wmask, v[7 - q].y, src));
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
   }
   p2_sync<WS>(wmask);
   if (valid) {
-    float2* X = a.X + r * H;
+    float2* X = a.X + r * a.xp;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       int k = j + q * T;
@@ -298,23 +298,18 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
 // Columns.  Block = TX columns x L/E threads; thread (j, c), c fastest, so a
 // warp reads whole row segments of TX consecutive columns.
 // ---------------------------------------------------------------------------
-enum { P2_Y_FWD = 0, P2_Y_INV = 1, P2_Z_BIN = 2, P2_Z_ADJ = 3 };
-
-// E: values per thread (ur_fast_col_e); threads per column block: 512, or 1024
-// for N >= 2048 so that a block still spans at least two columns (16-byte row
-// segments) of the half spectrum.  MINB: resident blocks per SM the register
-// budget is cut for (the z pass with binning fits in 32 registers: four blocks
-// of 512 threads; 16 values per thread take 64)
-template <int N, int MODE = P2_Y_FWD>
+// Threads per column block: 512, or 1024 for N >= 2048 so that a block still spans at least two
+// columns (16-byte row segments) of the half spectrum; 16 values per thread take 64 registers.
+template <int N>
 struct ColCfg {
-  static constexpr int E = UR_FAST_COL_E(N);
+  static constexpr int E = UR_FAST_COL_E;
   static constexpr int THREADS = N >= 2048 ? 1024 : 512;
   static constexpr int TX = THREADS / (N / E);
-  static constexpr int MINB = E == 16 ? 65536 / (64 * THREADS) : N >= 2048 ? 2 : MODE == P2_Z_BIN ? 4 : 3;
+  static constexpr int MINB = 65536 / (64 * THREADS);
 };
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS, (ColCfg<N, MODE>::MINB)) k_p2_cols(ColArgs a) {
+__global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols(ColArgs a) {
   // column pitch = 2 (mod 16) float2: the TX columns a warp touches fall on different banks
   constexpr int E = ColCfg<N>::E;
   constexpr int T = N / E, TX = ColCfg<N>::TX, PITCH = P2<N>::PITCH + 2, H = N / 2 + 1, M = N / 2;
@@ -595,7 +590,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
   const bool valid = y < N;
   for (int i = threadIdx.x; i < U; i += blockDim.x) acc[i] = 0.f;
   float2* line = sm + t * PITCH;
-  const float2* Yrow = a.Y + ((long long)(z - a.ybase_z) * N + (valid ? y : 0)) * H;
+  const float2* Yrow = a.Y + ((long long)(z - a.ybase_z) * N + (valid ? y : 0)) * a.yp;
   // all nine loads of the row (k = j + q T, and k = M) are issued together
   float2 ld[9];
 #pragma unroll
@@ -743,11 +738,8 @@ static ur_status launch_cols_n(int mode, const ColArgs& a, cudaStream_t s) {
 }
 
 ur_status ur_fast_cols(int n, int mode, const ColArgs& a, cudaStream_t s) {
+  if (ur_pair_supported(n)) return ur_pair_cols(n, mode, a, s);
   switch (n) {
-    case 64: return launch_cols_n<64>(mode, a, s);
-    case 128: return launch_cols_n<128>(mode, a, s);
-    case 256: return launch_cols_n<256>(mode, a, s);
-    case 512: return launch_cols_n<512>(mode, a, s);
     case 1024: return launch_cols_n<1024>(mode, a, s);
     case 2048: return launch_cols_n<2048>(mode, a, s);
     case 4096: return launch_cols_n<4096>(mode, a, s);

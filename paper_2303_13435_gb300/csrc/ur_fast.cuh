@@ -4,14 +4,17 @@
 #include "ur_forward.cuh"
 #include "ur_density.cuh"
 
-// Values per thread of the power-of-two column transforms of length n: 16 from 1024 on
-// (three radix-16 stages at 4096 instead of four radix-8 ones; measured 22-23 % faster
-// steps at 1024-4096), 8 below (16 was 17 % slower at 512: half the resident warps).
-#define UR_FAST_COL_E(n) ((n) >= 1024 ? 16 : 8)
+// Values per column and thread of the column transforms: 8 up to 512 (pairs of columns, ur_pair.cu),
+// 16 from 1024 on (single columns, ur_fast.cu: three radix-16 stages at 4096 instead of four radix-8
+// ones; measured 22-23 % faster steps).
+#define UR_FAST_COL_E 16
+
+enum { P2_Y_FWD = 0, P2_Y_INV = 1, P2_Z_BIN = 2, P2_Z_ADJ = 3 };
 
 struct RowArgs {
   const void* ed;          // density rows (GEN = 0), plane-major, nrows x N
-  float2* X;               // output half-spectrum rows, nrows x (N/2+1)
+  float2* X;               // output half-spectrum rows, nrows x (N/2+1), xp apart
+  int xp;
   long long nrows;
   int z0;                  // absolute plane index of row 0 / N (GEN = 1)
   const float* cell;       // GEN = 1: unit cell U^3
@@ -27,6 +30,7 @@ struct RowArgs {
 
 struct GradArgs {
   const float2* Y;         // inverse-transformed rows (along z and y), planes [ybase_z, ...)
+  int yp;                  // row pitch of Y
   int ybase_z;
   int z0;                  // first absolute plane of this launch
   int rb;                  // rows per block (set by the launcher)
@@ -53,4 +57,7 @@ struct BatchRowsItem {
 bool ur_fast_supported(int n);
 ur_status ur_fast_rows(int n, const RowArgs& a, int gen, int ed_f16, cudaStream_t s);
 ur_status ur_fast_cols(int n, int mode, const ColArgs& a, cudaStream_t s);
+bool ur_pair_supported(int n);
+size_t ur_pair_twiddles(int n, float4* out);
+ur_status ur_pair_cols(int n, int mode, const ColArgs& a, cudaStream_t s);
 ur_status ur_fast_rows_grad(int n, const GradArgs& a, int nplanes, cudaStream_t s);

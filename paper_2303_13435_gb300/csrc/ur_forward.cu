@@ -109,7 +109,7 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
     const float2 d = make_float2(0.5f * (zk.x - zc.x), 0.5f * (zk.y - zc.y));
     const float2 o = make_float2(d.y, -d.x);  // -i d
     const float2 w = __ldg(tw + k);
-    X[r * H + k] = cadd(e, cmul(w, o));
+    X[r * ra.xp + k] = cadd(e, cmul(w, o));
   }
 }
 
@@ -785,8 +785,8 @@ ur_status ur_configure_kernels(ur_plan* p) {
   UR_CUDA_CHECK(cudaMemcpy(p->d_sched, p->sched_n.st, sizeof(StageInfo) * UR_MAX_STAGES, cudaMemcpyHostToDevice));
   UR_CUDA_CHECK(cudaMemcpy(p->d_sched + UR_MAX_STAGES, p->sched_m.st, sizeof(StageInfo) * UR_MAX_STAGES, cudaMemcpyHostToDevice));
   // workspace regions
-  p->ws_inter = (size_t)p->nz * n * p->H * sizeof(float2);
-  p->ws_inv = (size_t)n * n * p->H * sizeof(float2);
+  p->ws_inter = (size_t)p->nz * n * p->xp * sizeof(float2);
+  p->ws_inv = (size_t)n * n * p->xp * sizeof(float2);
   p->ws_sigma = (size_t)p->nbins * sizeof(float);
   // host-resident ED: slabs of about 256 MiB, two of them in the workspace
   {
@@ -799,7 +799,7 @@ ur_status ur_configure_kernels(ur_plan* p) {
   }
   // out-of-core adjoint: about 4 GiB of inverse intermediate per slab
   {
-    long long ap = (long long)((4ull << 30) / ((size_t)n * p->H * sizeof(float2)));
+    long long ap = (long long)((4ull << 30) / ((size_t)n * p->xp * sizeof(float2)));
     if (ap < 1) ap = 1;
     if (ap > n) ap = n;
     p->adj_slab_planes = (int)ap;
@@ -860,7 +860,8 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
     RowArgs r = ra;
     r.stw = p->stw ? p->stw + p->stw_m_off : nullptr;
     r.fu = FastDiv((uint32_t)(ra.ucell > 0 ? ra.ucell : 1));
-    r.X = X + p0 * n * H;
+    r.X = X + p0 * n * p->xp;
+    r.xp = p->xp;
     r.nrows = np * n;
     r.z0 = ra.z0 + (int)p0;
     if (!gen) r.ed = (const char*)ra.ed + p0 * (long long)n * n * (p->ed_dtype == UR_F16 ? 2 : 4);
@@ -886,8 +887,8 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
     a.src = r.X;
     a.dst = r.X;
     a.ncols = np * H;
-    a.A = (long long)n * H;
-    a.S = H;
+    a.A = (long long)n * p->xp;
+    a.S = p->xp;
     a.Ad = a.A;
     a.Sd = a.S;
     a.nload = n;
@@ -926,8 +927,8 @@ ur_status ur_column_pass(const ur_plan* p, const float2* X, double* bins, float2
   ColArgs a = ur_col_args(p);
   a.src = X;
   a.ncols = (long long)p->n * p->H;
-  a.A = p->H;
-  a.S = (long long)p->n * p->H;
+  a.A = p->xp;
+  a.S = (long long)p->n * p->xp;
   a.nload = p->nz;
   a.zoff = p->z0;
   const double n3 = (double)p->n * p->n * p->n;

@@ -15,6 +15,7 @@ struct ColArgs {
   const float2* src;
   float2* dst;
   long long ncols;
+  int nouter;        // pair kernels, y passes: planes (set by the launcher)
   int N, H, M;
   long long A;       // source offset per outer index (c / H)
   long long S;       // source stride between column elements
@@ -57,6 +58,7 @@ struct ColArgs {
 // generic adjoint row pass (one block: a batch of rows wrapping onto one cell row)
 struct GenGradArgs {
   const float2* Y;
+  int yp;            // row pitch of Y
   int N, RB, nst;
   const StageInfo* sched;
   const float2* tw;

@@ -373,6 +373,14 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
   p->n = n;
   p->M = n / 2;
   p->H = n / 2 + 1;
+  // pair kernels: rows of the intermediates start on 32-byte boundaries, so their row segments are
+  // whole sectors (at 1024^3 the padding cost the adjoint z pass 5 %, so other grids keep N/2+1); a
+  // plan that fits the built-in scratch of ur_fft_intensity_noalloc only without the padding keeps
+  // rows of N/2+1 too
+  p->xp = ur_pair_supported(n) ? (p->H + 3) / 4 * 4 : p->H;
+  if ((size_t)g->nz * n * p->xp * sizeof(float2) > (size_t)UR_NOALLOC_SCRATCH_BYTES &&
+      (size_t)g->nz * n * p->H * sizeof(float2) <= (size_t)UR_NOALLOC_SCRATCH_BYTES)
+    p->xp = p->H;
   p->dx = g->dx;
   p->dq = 2.0 * M_PI / ((double)n * g->dx);
   p->ed_dtype = g->ed_dtype;
@@ -417,11 +425,14 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
   if (ur_fast_supported(n)) {
     int lg = 0;
     while ((1 << lg) < n) ++lg;
-    // columns (N points) run UR_FAST_COL_E(n) values per thread, rows (N/2 points) 8
-    const int ecol = UR_FAST_COL_E(n);
-    const size_t cn = stage_twiddles(lg, ecol, nullptr), cm = stage_twiddles(lg - 1, 8, nullptr);
+    // columns (N points): the pair table, or stages of UR_FAST_COL_E values per thread; rows (N/2
+    // points) 8
+    const bool pair = ur_pair_supported(n);
+    const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : stage_twiddles(lg, UR_FAST_COL_E, nullptr);
+    const size_t cm = stage_twiddles(lg - 1, 8, nullptr);
     float2* st_h = (float2*)malloc(sizeof(float2) * (cn + cm + 1));
-    stage_twiddles(lg, ecol, st_h);
+    if (pair) ur_pair_twiddles(n, (float4*)st_h);
+    else stage_twiddles(lg, UR_FAST_COL_E, st_h);
     stage_twiddles(lg - 1, 8, st_h + cn);
     p->stw_m_off = (int)cn;
     const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (cn + cm + 1));
@@ -520,7 +531,7 @@ extern "C" size_t ur_workspace_size(const ur_plan* p, int32_t what) {
     // fixed layout after the forward intermediate: [host staging slabs][Y slab][sigma][two dL/dm slabs]
     const size_t S = (size_t)p->adj_slab_planes;
     if (!(what & UR_WS_HOST_SLABS)) b += 2 * ur_align_up(p->ws_slab, 256);
-    b += ur_align_up(S * p->n * p->H * sizeof(float2), 256) + ur_align_up(p->ws_sigma, 256) +
+    b += ur_align_up(S * p->n * p->xp * sizeof(float2), 256) + ur_align_up(p->ws_sigma, 256) +
          2 * ur_align_up((size_t)ur_adj_dm_planes(p) * p->n * p->n * sizeof(float), 256);
   }
   return b;

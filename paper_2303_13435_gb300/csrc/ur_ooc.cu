@@ -23,7 +23,7 @@ extern "C" ur_status ur_plan_set_slab_planes(ur_plan* p, int32_t planes) {
 extern "C" ur_status ur_plan_set_chunk_planes(ur_plan* p, int32_t planes) {
   UR_REQUIRE(p && planes >= 1, "ur_plan_set_chunk_planes: bad argument");
   if (!p->fast) return UR_OK;
-  const size_t plane_bytes = (size_t)p->n * p->H * sizeof(float2);
+  const size_t plane_bytes = (size_t)p->n * p->xp * sizeof(float2);
   p->chunk_planes = planes > p->n ? p->n : planes;
   // whole-grid passes transform Y in place; chunks need their own buffer
   p->ws_chunk = p->chunk_planes < p->n ? (size_t)p->chunk_planes * plane_bytes : 0;
@@ -44,7 +44,7 @@ ur_status ur_fft_intensity_host(const ur_plan* p, const void* ed_host, double* b
                "ur_fft_intensity (host ED): ed must be page-locked host memory (cudaHostAlloc or registered)");
   }
   UR_TRY(ur_fault_point("fft_intensity"));
-  const int n = p->n, H = p->H;
+  const int n = p->n;
   const size_t esz = p->ed_dtype == UR_F16 ? 2 : 4;
   const size_t plane_bytes = (size_t)n * n * esz;
   const int S = p->slab_planes;
@@ -106,7 +106,7 @@ ur_status ur_fft_intensity_host(const ur_plan* p, const void* ed_host, double* b
       }
       cudaEventRecord(copy_done[b], cs);
       cudaStreamWaitEvent(s, copy_done[b], 0);
-      const ur_status ps = ur_plane_pass(p, slab[b], np, X + (size_t)p0 * n * H, s);
+      const ur_status ps = ur_plane_pass(p, slab[b], np, X + (size_t)p0 * n * p->xp, s);
       if (ps != UR_OK) {
         fail(ps);
         break;

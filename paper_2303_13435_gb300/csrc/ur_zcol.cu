@@ -3,9 +3,9 @@
 // plan selects with ur_plan_set_tma_zpass (the default is the compile-time
 // kernel of ur_fast.cu, measured faster at 512^3: 268 against 311 us).
 //
-// Work unit: a tile of 16 consecutive spectrum columns c = ky_index (N/2+1) + kx
-// (the intermediate X[p][ky][kx] seen as rows of N (N/2+1) columns, one row per
-// plane holding density).  One thread issues a TMA load of the tile's nz planes
+// Work unit: a tile of 16 consecutive spectrum columns c = ky_index xp + kx, xp the
+// row pitch of the intermediate (X[p][ky][kx] seen as rows of N xp columns, one row
+// per plane holding density; columns with kx > N/2 are padding and reach no bin).  One thread issues a TMA load of the tile's nz planes
 // into shared memory (128-byte swizzle) while the block works on the previous
 // tile (two stages, mbarrier completion, bounded waits).  The kernel is
 // persistent: one block per SM walks a list of tiles; tiles whose columns all
@@ -50,6 +50,7 @@ constexpr int ZC_STAGES = 1;  // one tile in flight per block; two blocks per SM
 constexpr uint32_t ZC_NAN_BITS = 0x7fc00000u;
 
 struct ZArgs {
+  int xp;                // row pitch of X
   int nz, z0;            // planes of X and the absolute plane of X's first plane
   int box_rows, nbox;    // TMA rows per box (a multiple of 8) and boxes per tile
   int stage_bytes;       // bytes of one stage buffer (a multiple of 1024)
@@ -168,8 +169,10 @@ __global__ void __launch_bounds__(ZC_THREADS, 2) k_zcol(const __grid_constant__ 
     }
     const int T = a.tiles ? __ldg(a.tiles + i) : i;
     const int col = T * ZC_TILE + jcol;
-    const int kyi = col / H, kx = col - kyi * H, ky = kyi < M ? kyi : kyi - N;
-    const int c2 = kx * kx + ky * ky;
+    const int kyi = col / a.xp, kxr = col - kyi * a.xp, ky = kyi < M ? kyi : kyi - N;
+    const bool pad = kxr >= H;
+    const int kx = pad ? 0 : kxr;
+    const int c2 = pad ? 1 << 29 : kx * kx + ky * ky;  // padding: beyond every threshold
     // first bin of this thread's chunk of |kz| (issued early; used after the transform)
     const int m0 = CH * t;
     int b0 = nb;
@@ -220,9 +223,10 @@ __global__ void __launch_bounds__(ZC_THREADS, 2) k_zcol(const __grid_constant__ 
     // natural order: kz = t + 16 q
 #pragma unroll
     for (int q = 0; q < A; ++q) xw[2 * (t + 16 * q) + cw] = v[q];
-    if (a.fout) {
+    if (a.fout && !pad) {
+      float2* f = a.fout + (long long)kyi * H + kx;
 #pragma unroll
-      for (int q = 0; q < A; ++q) a.fout[(long long)(t + 16 * q) * N * H + col] = cscale(v[q], a.fscale);
+      for (int q = 0; q < A; ++q) f[(long long)(t + 16 * q) * N * H] = cscale(v[q], a.fscale);
     }
     __syncwarp();
     {
@@ -419,7 +423,7 @@ ur_status ur_zcol_prepare(ur_plan* p) {
       tw[k1 * 16 + t] = make_float2((float)cos(ang), (float)(-sin(ang)));
     }
   // tiles with at least one column below the closing threshold
-  const long long ntile_all = (long long)n * H / ZC_TILE;
+  const long long ntile_all = (long long)n * p->xp / ZC_TILE;
   int32_t* tl = (int32_t*)malloc(sizeof(int32_t) * ntile_all);
   int cnt = 0;
   const int64_t tb = p->thr_host[p->nbins];
@@ -427,8 +431,8 @@ ur_status ur_zcol_prepare(ur_plan* p) {
     bool keep = false;
     for (int j = 0; j < ZC_TILE && !keep; ++j) {
       const long long c = T * ZC_TILE + j;
-      const int kyi = (int)(c / H), kx = (int)(c % H), ky = kyi < M ? kyi : kyi - n;
-      keep = (int64_t)kx * kx + (int64_t)ky * ky < tb;
+      const int kyi = (int)(c / p->xp), kx = (int)(c % p->xp), ky = kyi < M ? kyi : kyi - n;
+      keep = kx < H && (int64_t)kx * kx + (int64_t)ky * ky < tb;
     }
     if (keep) tl[cnt++] = (int32_t)T;
   }
@@ -463,8 +467,9 @@ static ur_status zcol_launch(const ur_plan* p, const CUtensorMap& tm, ZArgs a, c
 }
 
 static ur_status zcol_common(const ur_plan* p, const float2* X, ZArgs& a, CUtensorMap& tm) {
-  const int n = p->n, H = p->H;
+  const int n = p->n, xp = p->xp;
   memset(&a, 0, sizeof a);
+  a.xp = xp;
   a.nz = p->nz;
   a.z0 = p->z0;
   a.nbox = (p->nz + 255) / 256;
@@ -474,7 +479,7 @@ static ur_status zcol_common(const ur_plan* p, const float2* X, ZArgs& a, CUtens
   a.thr = p->thr;
   a.lut = p->binlut;
   a.nbins = p->nbins;
-  return ur_tmap_2d_u64(&tm, X, (uint64_t)n * H, (uint64_t)p->nz, (uint64_t)n * H * 8, ZC_TILE, (uint32_t)a.box_rows,
+  return ur_tmap_2d_u64(&tm, X, (uint64_t)n * xp, (uint64_t)p->nz, (uint64_t)n * xp * 8, ZC_TILE, (uint32_t)a.box_rows,
                         true);
 }
 
@@ -487,7 +492,7 @@ ur_status ur_zcol_forward(const ur_plan* p, const float2* X, double* bins, float
   UR_TRY(zcol_common(p, X, a, tm));
   const int nb = p->nbins;
   a.tiles = F_out ? nullptr : p->zc_tiles;
-  a.ntiles = F_out ? (int)((long long)p->n * p->H / ZC_TILE) : p->zc_ntiles;
+  a.ntiles = F_out ? (int)((long long)p->n * p->xp / ZC_TILE) : p->zc_ntiles;
   a.iscale = iscale;
   a.vs = p->vsinc;
   a.bins = bins;
