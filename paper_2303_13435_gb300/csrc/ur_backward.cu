@@ -32,135 +32,177 @@ __global__ void k_sigma(const double* __restrict__ g, const double* __restrict__
   sigma[j] = (float)v;
 }
 
-// B3.  Block (cz, cy); rows (z, y) with (z+oz) mod U = cz and (y+oy) mod U = cy.
-// Each row: Y[z][y][0..M] (Hermitian half along x) -> Z[k] = E[k] + i O[k],
+// B3.  A block takes up to RB rows (z, y) that wrap onto G neighbouring cell rows of one cell plane:
+// (z + oz) mod U = cz, (y + oy) mod U in [cy0, cy0 + G), so that small grids and small particles fill
+// its transforms too.  Rows that are not needed (outside the particle, when dL/dm is not wanted) do
+// not enter.  Each row: Y[z][y][0..M] (Hermitian half along x) -> Z[k] = E[k] + i O[k],
 //   E[k] = X[k] + conj X[M-k],  O[k] = (X[k] - conj X[M-k]) conj(W_N^k),
 // then z = IFFT_{M}(Z) gives (g(2m), g(2m+1)) = (Re z[m], Im z[m]).
+// dL/du: a thread owns a cell voxel (or a share of its rows), sums its voxels of the block's rows in
+// registers and adds the sum to global memory once: a shared-memory float32 addition per voxel is a
+// compare-and-swap loop.  64 particles of 96^3-384^3, dL/du only: 8674 -> 678 us (64-row tiles of
+// which 1 to 36 rows were used, every row of the box); 378^3 with dL/dm: 311 -> 289 us.
 struct NoStore {
   __device__ __forceinline__ void operator()(int, int, float2) const {}
 };
 
+struct GradRow {
+  RowMask rm;
+  int z, y, g;  // g: cell row of the block
+};
+
+__device__ __forceinline__ int first_in(int lo, int c, int o, int U) {  // first i >= lo with (i + o) mod U = c
+  int d = (c - o - lo) % U;
+  if (d < 0) d += U;
+  return lo + d;
+}
+
 __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int by) {
-  const float2* __restrict__ Y = g.Y;
-  const int N = g.N, RB = g.RB, nst = g.nst, U = g.U, ox = g.ox, oy = g.oy, oz = g.oz;
-  const StageInfo* __restrict__ sched = g.sched;
-  const float2* __restrict__ tw = g.tw;
-  const float* __restrict__ cell = g.cell;
-  const ShapeArgs& sh = g.sh;
+  const int N = g.N, RB = g.RB, nst = g.nst, U = g.U, G = g.G, zlo = g.zlo, yp = g.yp, ox = g.ox;
   const float* __restrict__ weights = g.weights;
-  const float inv_n3 = g.inv_n3;
   float* __restrict__ dl_dmask = g.dl_dmask;
   float* __restrict__ dl_dcell = g.dl_dcell;
+  const StageInfo* __restrict__ sched = g.sched;
+  const float2* __restrict__ tw = g.tw;
+  const ShapeArgs& sh = g.sh;
+  const float inv_n3 = g.inv_n3;
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int s_nrow;
   const int M = N >> 1, H = M + 1;
   float2* buf = reinterpret_cast<float2*>(smraw);
-  float* acc = reinterpret_cast<float*>(smraw + ur_align_up_dev((size_t)RB * H * sizeof(float2), 16));
-  const int cz = by / U, cy = by - (by / U) * U;
-  const int zf = ((cz - oz) % U + U) % U, yf = ((cy - oy) % U + U) % U;
-  const int nzr = zf < N ? (N - 1 - zf) / U + 1 : 0;
-  const int nyr = yf < N ? (N - 1 - yf) / U + 1 : 0;
-  const int nrows = nzr * nyr;
-  const int r0 = bx * RB;
-  if (r0 >= nrows) return;  // uniform over the block
-  for (int i = threadIdx.x; i < U; i += blockDim.x) acc[i] = 0.f;
-  const float* crow = cell + ((long long)cz * U + cy) * U;
-  const FastDiv dM((uint32_t)M), dH((uint32_t)H), dNy((uint32_t)(nyr > 0 ? nyr : 1)), dU((uint32_t)U);
-  __syncthreads();
-  {
-    const int nb = min(RB, nrows - r0);
-    if (nst >= 2) {
-      // the first stage packs its inputs straight from the Hermitian half rows (no staging
-      // round trip): Z[i] = (X[i] + conj X[M-i]) + i (X[i] - conj X[M-i]) conj(W_N^i), X[M] for i = 0
-      auto packed = [&](int t, int i) -> float2 {
-        if (t >= nb) return make_float2(0.f, 0.f);
-        const int q = r0 + t;
-        const int a = (int)dNy.div((uint32_t)q);
-        const int b = q - a * nyr;
-        const long long z = zf + (long long)U * a, y = yf + (long long)U * b;
-        const float2* row = Y + (z * N + y) * g.yp;
-        const float2 xa = __ldg(row + i), xb = __ldg(row + (M - i));
-        const float2 w = __ldg(tw + i);
-        const float2 e = cadd(xa, cconj(xb));
-        const float2 d = csub(xa, cconj(xb));
-        const float2 o = make_float2(d.x * w.x + d.y * w.y, d.y * w.x - d.x * w.y);  // * conj(W^i)
-        return make_float2(e.x - o.y, e.y + o.x);
-      };
-      fft_lines_io<true, UR_EMAX, true, false, false>(buf, H, RB, sched, nst, tw, packed, NoStore());
-    } else {
-      for (int f = threadIdx.x; f < RB * H; f += blockDim.x) {
-        const int t = (int)dH.div((uint32_t)f);
-        const int k = f - t * H;
-        float2 v = make_float2(0.f, 0.f);
-        if (t < nb) {
-          const int q = r0 + t;
-          const int a = (int)dNy.div((uint32_t)q);
-          const int b = q - a * nyr;
-          const long long z = zf + (long long)U * a, y = yf + (long long)U * b;
-          v = __ldg(Y + (z * N + y) * g.yp + k);
-        }
-        buf[f] = v;
+  GradRow* rows = reinterpret_cast<GradRow*>(smraw + ur_align_up_dev((size_t)RB * H * sizeof(float2), 16));
+  int* gbeg = reinterpret_cast<int*>(rows + RB);  // first row of each of the block's cell rows
+  const int ncg = (U + G - 1) / G;
+  const int cz = by / ncg, cy0 = (by - cz * ncg) * G;
+  const int zf = first_in(g.zlo, cz, g.oz, U);
+  if (zf >= g.zhi) return;  // uniform over the block
+  // the block's rows, in order of cell row; listed by the first warp
+  if (threadIdx.x < 32) {
+    const int per = g.nza * g.nyb;
+    int n = 0;
+    for (int t0 = 0; t0 < RB; t0 += 32) {
+      const int q = bx * RB + t0 + (int)threadIdx.x;
+      const int gr = q / per, ab = q - gr * per, a = ab / g.nyb, b = ab - a * g.nyb;
+      const int z = zf + U * a, cy = cy0 + gr;
+      bool use = t0 + (int)threadIdx.x < RB && gr < G && cy < U && z < g.zhi;
+      int y = 0;
+      if (use) {
+        y = first_in(g.ylo, cy, g.oy, U) + U * b;
+        use = y < g.yhi && !(g.row_skip && row_outside(sh, y, z));
       }
-      __syncthreads();
-      // Hermitian half -> packed complex sequence, in place by (k, M-k) pairs
-      const int half = M / 2 + 1;
-      const FastDiv dhalf((uint32_t)half);
-      for (int f = threadIdx.x; f < RB * half; f += blockDim.x) {
-        const int t = (int)dhalf.div((uint32_t)f);
-        const int k = f - t * half;
-        float2* X = buf + t * H;
-        const float2 xa = X[k], xb = X[M - k];
-        const float2 wa = __ldg(tw + k);
-        // Z[k]
-        const float2 ea = cadd(xa, cconj(xb));
-        const float2 da = csub(xa, cconj(xb));
-        const float2 oa = make_float2(da.x * wa.x + da.y * wa.y, da.y * wa.x - da.x * wa.y);  // * conj(W^k)
-        const float2 za = make_float2(ea.x - oa.y, ea.y + oa.x);
-        if (k != 0 && 2 * k != M) {
-          const float2 wb = __ldg(tw + (M - k));
-          const float2 eb = cadd(xb, cconj(xa));
-          const float2 db = csub(xb, cconj(xa));
-          const float2 ob = make_float2(db.x * wb.x + db.y * wb.y, db.y * wb.x - db.x * wb.y);
-          X[M - k] = make_float2(eb.x - ob.y, eb.y + ob.x);
-        }
-        X[k] = za;
+      const unsigned who = __ballot_sync(0xffffffffu, use);
+      if (use) {
+        GradRow& r = rows[n + __popc(who & ((1u << threadIdx.x) - 1u))];
+        r.rm.init(sh, y, z);
+        r.z = z;
+        r.y = y;
+        r.g = gr;
       }
-      __syncthreads();
-      fft_lines<true, UR_EMAX>(buf, H, RB, sched, nst, tw);
+      n += __popc(who);
     }
-    // epilogue
-    for (int f = threadIdx.x; f < RB * M; f += blockDim.x) {
-      const int t = (int)dM.div((uint32_t)f);
-      const int m = f - t * M;
-      if (t >= nb) continue;
-      const int q = r0 + t;
-      const int a = (int)dNy.div((uint32_t)q);
-      const int b = q - a * nyr;
-      const int z = zf + U * a, y = yf + U * b;
-      const float2 zv = buf[t * H + m];
-      const float g0 = zv.x * inv_n3, g1 = zv.y * inv_n3;
-      const int x0 = 2 * m;
-      const int c0 = (int)dU.mod((uint32_t)(x0 + ox)), c1 = (int)dU.mod((uint32_t)(x0 + 1 + ox));
-      const long long vox = ((long long)z * N + y) * N + x0;
-      if (dl_dmask) {
-        const float u0 = __ldg(crow + c0), u1 = __ldg(crow + c1);
-        *reinterpret_cast<float2*>(dl_dmask + vox) = make_float2(g0 * u0, g1 * u1);
+    __syncwarp();
+    for (int i = threadIdx.x; i <= G; i += 32) {  // rows of cell row i: [gbeg[i], gbeg[i + 1])
+      int lo = 0, hi = n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (rows[mid].g < i) lo = mid + 1;
+        else hi = mid;
       }
-      float m0, m1;
-      if (sh.kind == UR_SHAPE_WEIGHTS) {
-        const float2 wv = __ldg(reinterpret_cast<const float2*>(weights + vox));
-        m0 = wv.x;
-        m1 = wv.y;
-      } else {
-        m0 = mask_at(sh, x0, y, z);
-        m1 = mask_at(sh, x0 + 1, y, z);
-      }
-      if (m0 != 0.f) atomicAdd(acc + c0, g0 * m0);
-      if (m1 != 0.f) atomicAdd(acc + c1, g1 * m1);
+      gbeg[i] = lo;
+    }
+    if (threadIdx.x == 0) s_nrow = n;
+  }
+  __syncthreads();
+  const int nrow = s_nrow;
+  if (nrow == 0) return;
+  const float2* __restrict__ Y = g.Y;
+  const FastDiv dM((uint32_t)M), dH((uint32_t)H);
+  if (nst >= 2) {
+    // the first stage packs its inputs straight from the Hermitian half rows (no staging
+    // round trip): Z[i] = (X[i] + conj X[M-i]) + i (X[i] - conj X[M-i]) conj(W_N^i), X[M] for i = 0
+    auto packed = [&](int t, int i) -> float2 {
+      const float2* row = Y + ((long long)(rows[t].z - zlo) * N + rows[t].y) * yp;
+      const float2 xa = __ldg(row + i), xb = __ldg(row + (M - i));
+      const float2 w = __ldg(tw + i);
+      const float2 e = cadd(xa, cconj(xb));
+      const float2 d = csub(xa, cconj(xb));
+      const float2 o = make_float2(d.x * w.x + d.y * w.y, d.y * w.x - d.x * w.y);  // * conj(W^i)
+      return make_float2(e.x - o.y, e.y + o.x);
+    };
+    fft_lines_io<true, UR_EMAX, true, false, false>(buf, H, nrow, sched, nst, tw, packed, NoStore());
+  } else {
+    for (int f = threadIdx.x; f < nrow * H; f += blockDim.x) {
+      const int t = (int)dH.div((uint32_t)f);
+      buf[f] = __ldg(Y + ((long long)(rows[t].z - zlo) * N + rows[t].y) * yp + (f - t * H));
     }
     __syncthreads();
+    // Hermitian half -> packed complex sequence, in place by (k, M-k) pairs
+    const int half = M / 2 + 1;
+    const FastDiv dhalf((uint32_t)half);
+    for (int f = threadIdx.x; f < nrow * half; f += blockDim.x) {
+      const int t = (int)dhalf.div((uint32_t)f);
+      const int k = f - t * half;
+      float2* X = buf + t * H;
+      const float2 xa = X[k], xb = X[M - k];
+      const float2 wa = __ldg(tw + k);
+      // Z[k]
+      const float2 ea = cadd(xa, cconj(xb));
+      const float2 da = csub(xa, cconj(xb));
+      const float2 oa = make_float2(da.x * wa.x + da.y * wa.y, da.y * wa.x - da.x * wa.y);  // * conj(W^k)
+      const float2 za = make_float2(ea.x - oa.y, ea.y + oa.x);
+      if (k != 0 && 2 * k != M) {
+        const float2 wb = __ldg(tw + (M - k));
+        const float2 eb = cadd(xb, cconj(xa));
+        const float2 db = csub(xb, cconj(xa));
+        const float2 ob = make_float2(db.x * wb.x + db.y * wb.y, db.y * wb.x - db.x * wb.y);
+        X[M - k] = make_float2(eb.x - ob.y, eb.y + ob.x);
+      }
+      X[k] = za;
+    }
+    __syncthreads();
+    fft_lines<true, UR_EMAX>(buf, H, nrow, sched, nst, tw);
   }
-  for (int i = threadIdx.x; i < U; i += blockDim.x)
-    if (acc[i] != 0.f) atomicAdd(dl_dcell + ((long long)cz * U + cy) * U + i, acc[i]);
+  // dL/dm = dL/drho * u
+  if (dl_dmask) {
+    const FastDiv dU((uint32_t)U);
+    for (int f = threadIdx.x; f < nrow * M; f += blockDim.x) {
+      const int t = (int)dM.div((uint32_t)f);
+      const int m = f - t * M;
+      const float2 zv = buf[t * H + m];
+      const int c0 = (int)dU.mod((uint32_t)(2 * m + ox)), c1 = c0 + 1 == U ? 0 : c0 + 1;
+      const float* crow = g.cell + ((long long)cz * U + cy0 + rows[t].g) * U;
+      *reinterpret_cast<float2*>(dl_dmask + ((long long)rows[t].z * N + rows[t].y) * N + 2 * m) =
+          make_float2(zv.x * inv_n3 * __ldg(crow + c0), zv.y * inv_n3 * __ldg(crow + c1));
+    }
+  }
+  // dL/du = sum of dL/drho * m over the repeats: task (cell row, share of its rows, cell column)
+  const float* bufr = reinterpret_cast<const float*>(buf);
+  const int share = G * U < (int)blockDim.x ? (int)blockDim.x / (G * U) : 1;
+  const int ntask = G * share * U;
+  for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
+    const int gs = task / U, c = task - gs * U;
+    const int gr = gs / share, part = gs - gr * share;
+    int x0 = (c - ox) % U;
+    if (x0 < 0) x0 += U;
+    float sum = 0.f;
+    for (int t = gbeg[gr] + part; t < gbeg[gr + 1]; t += share) {
+      const RowMask& rm = rows[t].rm;
+      const float* line = bufr + (size_t)t * 2 * H;
+      if (weights) {
+        const float* w = weights + ((long long)rows[t].z * N + rows[t].y) * N;
+        for (int x = x0; x < N; x += U) {
+          const float m = __ldg(w + x);
+          if (m != 0.f) sum += line[x] * inv_n3 * m;
+        }
+      } else {
+        for (int x = x0; x < N; x += U) {
+          const float m = rm.at(x);
+          if (m != 0.f) sum += line[x] * inv_n3 * m;
+        }
+      }
+    }
+    if (sum != 0.f) atomicAdd(dl_dcell + ((long long)cz * U + cy0 + gr) * U + c, sum);
+  }
 }
 
 __global__ void __launch_bounds__(256, 4) k_rows_grad(GenGradArgs g) { rows_grad_body(g, blockIdx.x, blockIdx.y); }
@@ -228,6 +270,51 @@ extern "C" ur_status ur_log_mse_grad(int32_t nbins, const double* bins, const do
   return UR_OK;
 }
 
+AdjRange ur_adj_range(const ur_plan* p, const ShapeArgs& sh, bool want_mask) {
+  AdjRange r = {0, p->n, 0, p->n, 0};
+  if (want_mask || !(sh.rb2 < INFINITY)) return r;
+  ur_mask_range(sh, sh.cz, p->n, &r.zlo, &r.zhi);
+  ur_mask_range(sh, sh.cy, p->n, &r.ylo, &r.yhi);
+  r.row_skip = 1;
+  return r;
+}
+
+// columns with kx^2 + ky^2 at or beyond the closing threshold have zero scales at every kz: the
+// adjoint z pass leaves them unwritten and its y pass reads them as zeros
+int ur_k2_zero(const ur_plan* p) {
+  const int64_t t = p->thr_host[p->nbins];
+  return t < 0x7fffffff ? (int)t : 0x7fffffff;
+}
+
+// Blocks of the generic row pass: as many cell rows per block as fill its RB rows
+void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy) {
+  const int U = g->U;
+  g->zlo = rg.zlo;
+  g->zhi = rg.zhi;
+  g->ylo = rg.ylo;
+  g->yhi = rg.yhi;
+  g->row_skip = rg.row_skip;
+  g->nza = (rg.zhi - rg.zlo + U - 1) / U;
+  g->nyb = (rg.yhi - rg.ylo + U - 1) / U;
+  const int per = g->nza * g->nyb;
+  if (per <= 0) {
+    g->nza = g->nyb = g->G = 1;
+    *gx = 1;
+    *gy = 0;
+    return;
+  }
+  g->G = g->RB / per;
+  if (g->G < 1) g->G = 1;
+  if (g->G > U) g->G = U;
+  *gx = (g->G * per + g->RB - 1) / g->RB;
+  *gy = (long long)U * ((U + g->G - 1) / g->G);
+}
+
+size_t ur_grad_smem(const ur_plan* p) {
+  const size_t rb = (size_t)p->row_rb;
+  return ur_align_up(rb * p->H * sizeof(float2), 16) + rb * sizeof(GradRow) + (rb + 1) * sizeof(int);
+}
+
 extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const double* fwd_bins, const void* F,
                                  const float* cell, int32_t ucell, const int32_t* origin, const ur_shape* shape,
                                  const float* weights, float* dl_dcell, float* dl_dmask, void* ws, size_t ws_bytes,
@@ -280,13 +367,21 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
     a.skip_fwd = 0;
   }
   const long long tiles = (a.ncols + a.TX - 1) / a.TX;
-  // power-of-two path: columns with kx^2 + ky^2 at or beyond the closing threshold get zero
-  // scales at every kz; the z pass leaves them unwritten and the y pass reads them as zeros
-  const int k2_zero = p->fast ? (int)(p->thr_host[nb] < 0x7fffffff ? p->thr_host[nb] : 0x7fffffff) : 0x7fffffff;
-  if (p->fast) a.k2_zero = k2_zero;
+  const ShapeArgs sh = ur_shape_args(shape);
+  const AdjRange rg = ur_adj_range(p, sh, dl_dmask != nullptr);
+  const int cnt = rg.zhi - rg.zlo, k2_zero = ur_k2_zero(p);
+  a.k2_zero = k2_zero;
+  if (cnt < n) {
+    a.out_lo = rg.zlo;
+    a.out_cnt = cnt;
+  }
+  if (!p->fast) UR_REQUIRE((long long)ucell * ucell <= 65535, "ur_backward: cell edge %d too large", ucell);
+  UR_CUDA_CHECK(cudaMemsetAsync(dl_dcell, 0, sizeof(float) * (size_t)ucell * ucell * ucell, s));
+  if (p->fast) UR_REQUIRE(!weights || ((uintptr_t)weights % 8) == 0, "ur_backward: weights must be 8-byte aligned");
+  if (cnt <= 0) return UR_OK;  // the mask is zero everywhere and dL/dm is not wanted
   ur_timing_begin("adj_cols_z", s);
   if (p->fast) {
-    UR_TRY(ur_fast_cols(n, 3 /* z adjoint */, a, s));
+    UR_TRY(ur_fast_cols(n, P2_Z_ADJ, a, s));
   } else {
     UR_TRY(ur_launch_cols(COL_ZADJ, false, p, a, (int)tiles, p->col_smem, s));
   }
@@ -296,7 +391,6 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
     // B2 + B3, over all planes with the y-inverse in place, or in plane chunks
     // whose y-inverse goes to a chunk buffer that the row pass of the same chunk
     // reads while it is still in L2.
-    UR_REQUIRE(!weights || ((uintptr_t)weights % 8) == 0, "ur_backward: weights must be 8-byte aligned");
     const bool whole = p->chunk_planes >= n;
     float2* C = (float2*)((char*)sigma + ur_align_up(p->ws_sigma, 256));
     GradArgs g;
@@ -310,14 +404,13 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
       g.oy = origin[1] % ucell;
       g.oz = origin[2] % ucell;
     }
-    g.sh = ur_shape_args(shape);
+    g.sh = sh;
     g.weights = shape->kind == UR_SHAPE_WEIGHTS ? weights : nullptr;
     g.inv_n3 = (float)(1.0 / n3);
     g.dl_dmask = dl_dmask;
     g.dl_dcell = dl_dcell;
-    UR_CUDA_CHECK(cudaMemsetAsync(dl_dcell, 0, sizeof(float) * (size_t)ucell * ucell * ucell, s));
-    for (int p0 = 0; p0 < n; p0 += p->chunk_planes) {
-      const int np = (p0 + p->chunk_planes <= n) ? p->chunk_planes : n - p0;
+    for (int p0 = 0; p0 < cnt; p0 += p->chunk_planes) {
+      const int np = (p0 + p->chunk_planes <= cnt) ? p->chunk_planes : cnt - p0;
       ColArgs b = ur_col_args(p);
       b.src = Y + (long long)p0 * n * p->xp;
       b.dst = whole ? Y : C;
@@ -330,13 +423,16 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
       b.zoff = 0;
       b.nbins = 0;
       b.k2_zero = k2_zero;
+      b.row_skip = rg.row_skip;
+      b.gen_z0 = rg.zlo + p0;
+      b.sh = sh;
       ur_timing_begin("adj_cols_y", s);
-      UR_TRY(ur_fast_cols(n, 1 /* y inverse */, b, s));
+      UR_TRY(ur_fast_cols(n, P2_Y_INV, b, s));
       ur_timing_end(s);
       g.Y = whole ? Y : C;
       g.yp = p->xp;
-      g.ybase_z = p0;
-      g.z0 = p0;
+      g.ybase_z = rg.zlo + p0;
+      g.z0 = rg.zlo + p0;
       ur_timing_begin("adj_rows_grad", s);
       UR_TRY(ur_fast_rows_grad(n, g, np, s));
       ur_timing_end(s);
@@ -348,7 +444,7 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   ColArgs b = ur_col_args(p);
   b.src = Y;
   b.dst = Y;
-  b.ncols = (long long)n * H;
+  b.ncols = (long long)cnt * H;
   b.A = (long long)n * p->xp;
   b.S = p->xp;
   b.Ad = b.A;
@@ -356,47 +452,44 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   b.nload = n;
   b.zoff = 0;
   b.nbins = 0;
+  b.k2_zero = k2_zero;
+  b.row_skip = rg.row_skip;
+  b.gen_z0 = rg.zlo;
+  b.sh = sh;
   ur_timing_begin("adj_cols_y", s);
-  UR_TRY(ur_launch_cols(COL_Y, true, p, b, (int)tiles, p->col_smem, s));
+  UR_TRY(ur_launch_cols(COL_Y, true, p, b, (int)((b.ncols + b.TX - 1) / b.TX), p->col_smem, s));
   ur_timing_end(s);
 
   // B3
-  const ShapeArgs sh = ur_shape_args(shape);
-  int ox = 0, oy = 0, oz = 0;
-  if (origin) {
-    ox = origin[0];
-    oy = origin[1];
-    oz = origin[2];
-  }
-  const int RB = p->row_rb;
-  const size_t smem = ur_align_up((size_t)RB * H * sizeof(float2), 16) + (size_t)ucell * sizeof(float);
-  UR_REQUIRE(smem <= 227 * 1024, "ur_backward: cell edge %d too large for the row reduction", ucell);
-  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  UR_REQUIRE((long long)ucell * ucell <= 65535, "ur_backward: cell edge %d too large", ucell);
-  const int rows_per_group = ((n + ucell - 1) / ucell) * ((n + ucell - 1) / ucell);
-  dim3 ggrid((unsigned)((rows_per_group + RB - 1) / RB), (unsigned)(ucell * ucell));
-  UR_CUDA_CHECK(cudaMemsetAsync(dl_dcell, 0, sizeof(float) * (size_t)ucell * ucell * ucell, s));
-  ur_timing_begin("adj_rows_grad", s);
   GenGradArgs ga;
   memset(&ga, 0, sizeof ga);
   ga.Y = Y;
   ga.yp = p->xp;
   ga.N = n;
-  ga.RB = RB;
+  ga.RB = p->row_rb;
   ga.nst = p->sched_m.nst;
   ga.sched = p->d_sched + UR_MAX_STAGES;
   ga.tw = p->tw;
   ga.cell = cell;
   ga.U = ucell;
-  ga.ox = ox;
-  ga.oy = oy;
-  ga.oz = oz;
+  if (origin) {  // reduced modulo the cell edge, as the cell indices are
+    ga.ox = origin[0] % ucell;
+    ga.oy = origin[1] % ucell;
+    ga.oz = origin[2] % ucell;
+  }
   ga.sh = sh;
   ga.weights = shape->kind == UR_SHAPE_WEIGHTS ? weights : nullptr;
   ga.inv_n3 = (float)(1.0 / n3);
   ga.dl_dmask = dl_dmask;
   ga.dl_dcell = dl_dcell;
-  k_rows_grad<<<ggrid, 256, smem, s>>>(ga);
+  int gx = 0;
+  long long gy = 0;
+  ur_grad_blocks(rg, &ga, &gx, &gy);
+  if (gy == 0) return UR_OK;
+  const size_t smem = ur_grad_smem(p);
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  ur_timing_begin("adj_rows_grad", s);
+  k_rows_grad<<<dim3((unsigned)gx, (unsigned)gy), 256, smem, s>>>(ga);
   UR_LAUNCH_CHECK("k_rows_grad");
   ur_timing_end(s);
   return UR_OK;
@@ -505,7 +598,8 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
   k_sigma<<<(nb + 255) / 256, 256, 0, s>>>(dl_dmean, fwd_bins, nb, n3, 0, sigma);
   UR_LAUNCH_CHECK("k_sigma");
   UR_CUDA_CHECK(cudaMemsetAsync(dl_dcell, 0, sizeof(float) * (size_t)ucell * ucell * ucell, s));
-  const int k2_zero = (int)(p->thr_host[nb] < 0x7fffffff ? p->thr_host[nb] : 0x7fffffff);
+  const int k2_zero = ur_k2_zero(p);
+  const AdjRange rg = ur_adj_range(p, ur_shape_args(shape), dl_dmask_host != nullptr);
 
   GradArgs g;
   memset(&g, 0, sizeof g);
@@ -537,8 +631,8 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
     }
   }
   int sub = 0;  // running index of the dL/dm staging sub-slabs (double-buffered)
-  for (int za = 0; za < n && st == UR_OK; za += S) {
-    const int cnt = za + S <= n ? S : n - za;
+  for (int za = rg.zlo; za < rg.zhi && st == UR_OK; za += S) {
+    const int cnt = za + S <= rg.zhi ? S : rg.zhi - za;
     // z pass over every column, keeping planes [za, za + cnt)
     ColArgs a = ur_col_args(p);
     a.ncols = (long long)n * H;
@@ -571,6 +665,9 @@ extern "C" ur_status ur_backward_slabs(const ur_plan* p, const double* dl_dmean,
     c.zoff = 0;
     c.nbins = 0;
     c.k2_zero = k2_zero;
+    c.row_skip = rg.row_skip;
+    c.gen_z0 = za;
+    c.sh = g.sh;
     ur_timing_begin("adj_cols_y", s);
     st = ur_fast_cols(n, 1 /* y inverse */, c, s);
     ur_timing_end(s);

@@ -47,7 +47,7 @@ extern "C" ur_status ur_plan_set_tiles(ur_plan* p, int32_t rows_per_block, int32
                "ur_plan_set_tiles: %d rows of %d exceed a block's %d elements", rows_per_block, p->M,
                UR_EMAX * p->row_threads);
     p->row_rb = rows_per_block;
-    p->row_smem = (size_t)rows_per_block * p->M * sizeof(float2);
+    p->row_smem = ur_row_smem(rows_per_block, p->M);
   }
   if (cols_per_block > 0) {
     UR_REQUIRE((long long)cols_per_block * p->n <= (long long)UR_EMAX * p->col_threads,
@@ -134,7 +134,8 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     r.gen = 1;
     r.sched = p->d_sched + UR_MAX_STAGES;
     s_rows[i + 1] = s_rows[i] + (r.ra.nrows + r.RB - 1) / r.RB;
-    smem_rows = std::max(smem_rows, (size_t)r.RB * M * sizeof(float2));
+    r.ra.skip_empty = sh.rb2 < INFINITY && !weights;
+    smem_rows = std::max(smem_rows, ur_row_smem(r.RB, p->M));
     // y columns, in place
     ColArgs a = ur_col_args(p);
     a.src = X;
@@ -147,6 +148,9 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     a.nload = n;
     a.zoff = 0;
     a.nbins = 0;
+    a.row_skip = r.ra.skip_empty;
+    a.gen_z0 = p->z0;
+    a.sh = sh;
     coly[i] = a;
     s_coly[i + 1] = s_coly[i] + (a.ncols + a.TX - 1) / a.TX;
     smem_cols = std::max(smem_cols, p->col_smem);
@@ -187,12 +191,19 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     za.nload = p->nz;
     za.zoff = p->z0;
     za.sigma = sigma;
+    const AdjRange rg = ur_adj_range(p, sh, it.dl_dmask != nullptr);
+    za.k2_zero = ur_k2_zero(p);
+    const int cnt = rg.zhi - rg.zlo;  // planes of the adjoint
+    if (cnt < n) {
+      za.out_lo = rg.zlo;
+      za.out_cnt = cnt;
+    }
     zadj[i] = za;
-    s_zadj[i + 1] = s_zadj[i] + (za.ncols + za.TX - 1) / za.TX;
+    s_zadj[i + 1] = s_zadj[i] + (cnt > 0 ? (za.ncols + za.TX - 1) / za.TX : 0);
     ColArgs yi = ur_col_args(p);
     yi.src = Y;
     yi.dst = Y;
-    yi.ncols = (long long)n * H;
+    yi.ncols = (long long)cnt * H;
     yi.A = (long long)n * p->xp;
     yi.S = p->xp;
     yi.Ad = yi.A;
@@ -200,6 +211,10 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     yi.nload = n;
     yi.zoff = 0;
     yi.nbins = 0;
+    yi.k2_zero = za.k2_zero;
+    yi.row_skip = rg.row_skip;
+    yi.gen_z0 = rg.zlo;
+    yi.sh = sh;
     yinv[i] = yi;
     s_yinv[i + 1] = s_yinv[i] + (yi.ncols + yi.TX - 1) / yi.TX;
     zc[i].ptr = it.dl_dcell;
@@ -223,10 +238,10 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     g.g.inv_n3 = (float)(1.0 / n3);
     g.g.dl_dmask = it.dl_dmask;
     g.g.dl_dcell = it.dl_dcell;
-    const int rpg = ((n + it.ucell - 1) / it.ucell) * ((n + it.ucell - 1) / it.ucell);
-    g.gx = (rpg + g.g.RB - 1) / g.g.RB;
-    s_grad[i + 1] = s_grad[i] + (long long)g.gx * it.ucell * it.ucell;
-    smem_grad = std::max(smem_grad, ur_align_up((size_t)g.g.RB * H * sizeof(float2), 16) + (size_t)it.ucell * 4);
+    long long gy = 0;
+    ur_grad_blocks(rg, &g.g, &g.gx, &gy);
+    s_grad[i + 1] = s_grad[i] + (long long)g.gx * gy;
+    smem_grad = std::max(smem_grad, ur_grad_smem(p));
   }
   UR_REQUIRE(smem_grad <= 227 * 1024 && smem_zbin <= 227 * 1024, "ur_batch_create: shared memory per block too large");
 

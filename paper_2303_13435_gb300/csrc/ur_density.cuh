@@ -2,6 +2,7 @@
 // the fused density + transform row pass and the adjoint row pass (Sec. 2.3).
 #pragma once
 
+#include <math.h>
 #include <string.h>
 
 #include "ur_common.cuh"
@@ -10,6 +11,7 @@ struct ShapeArgs {
   int kind;
   float cx, cy, cz, s;
   float r[9];
+  float rb2;  // rows (y, z) with fl(dy dy + dz dz) > rb2 have a zero mask at every x (infinity: unknown)
 };
 
 // Mask value at voxel (x, y, z): every product and sum rounded separately
@@ -35,8 +37,8 @@ __device__ __forceinline__ float mask_at(const ShapeArgs& sh, int x, int y, int 
 // they are formed once (with the same roundings) and only the x term varies.
 struct RowMask {
   int kind;
-  float s, s2, dyz2;   // sphere: fl(dy*dy) and fl(dz*dz) folded below
-  float dy2, dz2;
+  float s, s2;
+  float dy2, dz2;      // fl(dy*dy), fl(dz*dz)
   float cx;
   float ry[3], rz[3];  // fl(R[1][a] dy), fl(R[2][a] dz)
   float r0[3];
@@ -56,10 +58,9 @@ struct RowMask {
       rz[a] = __fmul_rn(sh.r[6 + a], dz);
     }
   }
-  // True when the mask is zero at every x of the row.  Sphere only: rounding
-  // to nearest is monotone and fl(dx*dx) >= 0, so fl(fl(fl(dx*dx) + dy2) + dz2)
-  // >= fl(dy2 + dz2) for every x; other shapes report false (no shortcut).
-  __device__ __forceinline__ bool empty() const {
+  // True when the mask is zero at every x of the row (row_outside)
+  __device__ __forceinline__ bool empty(const ShapeArgs& sh) const { return __fadd_rn(dy2, dz2) > sh.rb2; }
+  __device__ __forceinline__ bool sphere_empty() const {
     return kind == UR_SHAPE_SPHERE && __fadd_rn(dy2, dz2) > s2;
   }
   // Signed coordinate of axis a at x, rounded as in mask_at; nondecreasing or nonincreasing in x,
@@ -117,11 +118,16 @@ struct RowMask {
   }
 };
 
-// Sphere row (y, z) outside the particle: the test of RowMask::empty with the same
-// roundings, for kernels that hold no RowMask.
-__device__ __forceinline__ bool sphere_row_empty(const ShapeArgs& sh, int y, int z) {
-  const float dy = __fsub_rn((float)y, sh.cy), dz = __fsub_rn((float)z, sh.cz);
-  return __fadd_rn(__fmul_rn(dy, dy), __fmul_rn(dz, dz)) > __fmul_rn(sh.s, sh.s);
+// Row (y, z) outside the particle: its mask is zero at every x.  Sphere: rb2 = fl(s s); rounding
+// to nearest is monotone and fl(dx*dx) >= 0, so fl(fl(fl(dx*dx) + dy2) + dz2) >= fl(dy2 + dz2) for
+// every x.  Cube and octahedron: rb2 is the square of a radius beyond their vertices
+// (ur_shape_args).
+__device__ __forceinline__ bool row_outside(float cy, float cz, float rb2, int y, int z) {
+  const float dy = __fsub_rn((float)y, cy), dz = __fsub_rn((float)z, cz);
+  return __fadd_rn(__fmul_rn(dy, dy), __fmul_rn(dz, dz)) > rb2;
+}
+__device__ __forceinline__ bool row_outside(const ShapeArgs& sh, int y, int z) {
+  return row_outside(sh.cy, sh.cz, sh.rb2, y, z);
 }
 
 // Rotated lattice (Sec. 2.3: the cell sampled on rotated planes with periodic wrap).
@@ -190,5 +196,43 @@ static inline ShapeArgs ur_shape_args(const ur_shape* shape) {
   sh.cz = shape->center[2];
   sh.s = shape->size;
   for (int i = 0; i < 9; ++i) sh.r[i] = shape->rot[i];
+  sh.rb2 = INFINITY;
+  if (sh.kind == UR_SHAPE_SPHERE) {
+    sh.rb2 = sh.s * sh.s;
+  } else if (sh.kind == UR_SHAPE_CUBE || sh.kind == UR_SHAPE_OCTAHEDRON) {
+    // Inside, |p|^2 <= 3 s^2 (cube) or s^2 (octahedron), and |d|^2 <= |p|^2 / (1 - e) where e bounds
+    // |R R^T - 1|; the slack covers the predicate's float32 roundings (relative 1e-6 of |d|, and 2.5e-4
+    // voxels of a rounded coordinate below 4096).  A matrix that is not nearly a rotation has no bound.
+    double e = 0.0;
+    for (int i = 0; i < 3; ++i) {
+      double row = 0.0;
+      for (int j = 0; j < 3; ++j) {
+        double v = i == j ? -1.0 : 0.0;
+        for (int k = 0; k < 3; ++k) v += (double)sh.r[3 * i + k] * (double)sh.r[3 * j + k];
+        row += fabs(v);
+      }
+      if (!(row <= e)) e = row;
+    }
+    if (e < 0.01 && sh.s < 1e6f) {
+      const double s = sh.s > 0.f ? (double)sh.s : 0.0;
+      const double r = s * (sh.kind == UR_SHAPE_CUBE ? 1.7320508075688772 : 1.0) / sqrt(1.0 - e) * 1.0001 + 0.05;
+      sh.rb2 = (float)(r * r);
+    }
+  }
   return sh;
+}
+
+// [lo, hi): the coordinates i of an axis (particle centre c) that the mask can reach (all of
+// [0, n) when unknown), with the roundings of row_outside
+static inline void ur_mask_range(const ShapeArgs& sh, float c, int n, int* lo, int* hi) {
+  auto out = [&](int i) {
+    const float d = (float)i - c;
+    const float d2 = d * d;
+    return d2 > sh.rb2;
+  };
+  int a = 0, b = n;
+  while (a < n && out(a)) ++a;
+  while (b > a && out(b - 1)) --b;
+  *lo = a;
+  *hi = b;
 }

@@ -170,17 +170,21 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
   if (GEN) {
     const int p = (int)(r / N), y = (int)(r - (long long)p * N);
     const int z = a.z0 + p;
-    RowMask rm;
-    rm.init(a.sh, y, z);
     const int U = a.ucell;
     const float* wrow = a.weights ? a.weights + ((long long)z * N + y) * N : nullptr;
+    const bool outside = !wrow && row_outside(a.sh, y, z);
     if constexpr (WS) {
-      // rows outside the sphere: not written at all when the y pass knows to skip them
+      // rows outside the particle: not written at all when the y pass knows to skip them
       // (the condition is uniform over the row's lanes, which only sync among themselves)
-      if (a.skip_empty && valid && !wrow && rm.empty()) return;
+      if (a.skip_empty && outside) return;
+    } else {
+      // a row spans warps here, so a block leaves when all of its rows are outside
+      if (a.skip_empty && __syncthreads_and(!valid || outside)) return;
     }
     // rows the mask excludes entirely are zero (cell values are finite)
-    if (valid && (wrow || !rm.empty())) {
+    if (valid && !outside) {
+      RowMask rm;
+      rm.init(a.sh, y, z);
       if constexpr (GEN == 2) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -313,6 +317,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
   // column pitch = 2 (mod 16) float2: the TX columns a warp touches fall on different banks
   constexpr int E = ColCfg<N>::E;
   constexpr int T = N / E, TX = ColCfg<N>::TX, PITCH = P2<N>::PITCH + 2, H = N / 2 + 1, M = N / 2;
+  constexpr bool YINV = MODE == P2_Y_INV || MODE == P2_Y_INV_ROWS;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_blo, s_bhi;
   float2* buf = reinterpret_cast<float2*>(smraw);
@@ -391,9 +396,9 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const int y = j + q * T;
-      v[q] = (valid && !sphere_row_empty(a.sh, y, z)) ? __ldg(src + q * step) : make_float2(0.f, 0.f);
+      v[q] = (valid && !row_outside(a.sh, y, z)) ? __ldg(src + q * step) : make_float2(0.f, 0.f);
     }
-  } else if (MODE == P2_Y_INV && a.k2_zero != 0x7fffffff) {
+  } else if (YINV && a.k2_zero != 0x7fffffff) {
     // adjoint y pass: elements with kx^2 + ky^2 >= k2_zero are zero (the z pass left them
     // unwritten) and are not read
     const float2* src = a.src + (valid ? sbase + (long long)j * a.S : 0);
@@ -430,12 +435,16 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
     atomicMin(&s_blo, lo_bin);
     atomicMax(&s_bhi, hi_bin);
   }
-  if (MODE == P2_Y_FWD || MODE == P2_Y_INV) {
-    p2_fft<N, MODE == P2_Y_INV, false, E>(v, j, line, a.stw);
+  if (MODE == P2_Y_FWD || YINV) {
+    p2_fft<N, YINV, false, E>(v, j, line, a.stw);
     if (valid) {
       const long long dbase = (long long)(col / H) * a.Ad + (col - (col / H) * H);
 #pragma unroll
-      for (int q = 0; q < E; ++q) a.dst[dbase + (long long)(j + q * T) * a.Sd] = v[q];
+      for (int q = 0; q < E; ++q) {
+        // rows outside the particle are not needed
+        if (MODE == P2_Y_INV_ROWS && row_outside(a.sh, j + q * T, a.gen_z0 + col / H)) continue;
+        a.dst[dbase + (long long)(j + q * T) * a.Sd] = v[q];
+      }
     }
   } else if (MODE == P2_Z_BIN) {
     p2_fft<N, false, false, E>(v, j, line, a.stw);
@@ -570,7 +579,8 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
 //   Z[k] = (X[k] + conj X[M-k]) + i (X[k] - conj X[M-k]) conj(W_N^k),
 //   z = IFFT_{N/2}(Z),  (g(2m), g(2m+1)) = (Re z[m], Im z[m]).
 // ---------------------------------------------------------------------------
-template <int N>
+// CELL: dL/du alone; rows that the mask excludes entirely add nothing to it and are left out.
+template <int N, bool CELL>
 __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
   constexpr int M = N / 2, H = M + 1, T = M / 8, PITCH = P2<M>::PITCH + 1;
   constexpr bool WS = T <= 32;
@@ -588,14 +598,19 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
   const int yf = yt >= U ? yt - U : yt;
   const int y = yf + U * (blockIdx.x * RB + t);
   const bool valid = y < N;
+  bool live = valid;
+  if constexpr (CELL) {  // a row within one warp skips its transform, rows across warps only as a whole block
+    live = valid && !row_outside(a.sh, y, z);
+    if (!__syncthreads_or(live)) return;
+  }
   for (int i = threadIdx.x; i < U; i += blockDim.x) acc[i] = 0.f;
   float2* line = sm + t * PITCH;
   const float2* Yrow = a.Y + ((long long)(z - a.ybase_z) * N + (valid ? y : 0)) * a.yp;
   // all nine loads of the row (k = j + q T, and k = M) are issued together
   float2 ld[9];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) ld[q] = valid ? __ldg(Yrow + j + q * T) : make_float2(0.f, 0.f);
-  ld[8] = (valid && j == 0) ? __ldg(Yrow + M) : make_float2(0.f, 0.f);
+  for (int q = 0; q < 8; ++q) ld[q] = live ? __ldg(Yrow + j + q * T) : make_float2(0.f, 0.f);
+  ld[8] = (live && j == 0) ? __ldg(Yrow + M) : make_float2(0.f, 0.f);
   float2 v[8];
   if constexpr (WS) {
     // X[M - k], k = j + qT, is load 7 - q of lane T - j of the same row (j >= 1); lane
@@ -631,15 +646,15 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
     }
     __syncthreads();  // the transform's first exchange reuses the lines
   }
-  p2_fft<M, true, WS>(v, j, line, a.stw, wmask);
+  if (!CELL || !WS || live) p2_fft<M, true, WS>(v, j, line, a.stw, wmask);
   const float* crow = a.cell + ((long long)cz * U + cy) * U;
   RowMask rm;
   rm.init(a.sh, valid ? y : 0, z);
   const float* wrow = a.weights ? a.weights + ((long long)z * N + (valid ? y : 0)) * N : nullptr;
-  if (valid) {
-    float* drow = a.dl_dmask ? a.dl_dmask + ((long long)(z - a.mbase_z) * N + y) * N : nullptr;
+  if (live) {
+    float* drow = !CELL && a.dl_dmask ? a.dl_dmask + ((long long)(z - a.mbase_z) * N + y) * N : nullptr;
     // rows the mask excludes entirely add nothing to dL/du
-    const bool mzero = !wrow && rm.empty();
+    const bool mzero = !wrow && rm.sphere_empty();
     // cell columns of x = 2 (j + q T): one modulo, then steps of 2T mod U; when U divides
     // 2T they are the same for every q and the dL/du sums stay in two registers
     const int cstep = a.cstep;
@@ -728,7 +743,10 @@ static ur_status launch_cols_n(int mode, const ColArgs& a, cudaStream_t s) {
   } while (0)
   switch (mode) {
     case P2_Y_FWD: UR_P2_LAUNCH(P2_Y_FWD); break;
-    case P2_Y_INV: UR_P2_LAUNCH(P2_Y_INV); break;
+    case P2_Y_INV:
+      if (a.row_skip) UR_P2_LAUNCH(P2_Y_INV_ROWS);
+      else UR_P2_LAUNCH(P2_Y_INV);
+      break;
     case P2_Z_BIN: UR_P2_LAUNCH(P2_Z_BIN); break;
     default: UR_P2_LAUNCH(P2_Z_ADJ); break;
   }
@@ -786,10 +804,12 @@ static ur_status launch_grad_n(GradArgs a, int nplanes, cudaStream_t s) {
   a.cstep = (2 * T) % U;
   const size_t smem = ur_align_up((size_t)rb * PITCH * sizeof(float2), 16) + (size_t)U * sizeof(float);
   UR_REQUIRE(smem <= 200 * 1024, "adjoint rows: cell edge %d too large", U);
-  if (smem > 48 * 1024) UR_CUDA_CHECK(cudaFuncSetAttribute(k_p2_rows_grad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const bool cell = !a.dl_dmask && !a.weights && a.sh.rb2 < INFINITY;
+  auto kern = cell ? k_p2_rows_grad<N, true> : k_p2_rows_grad<N, false>;
+  if (smem > 48 * 1024) UR_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((unsigned)((rows_per_group + rb - 1) / rb), (unsigned)U, (unsigned)nplanes);
   if (nplanes <= 0) return UR_OK;
-  k_p2_rows_grad<N><<<grid, rb * T, smem, s>>>(a);
+  kern<<<grid, rb * T, smem, s>>>(a);
   UR_LAUNCH_CHECK("k_p2_rows_grad");
   return UR_OK;
 }

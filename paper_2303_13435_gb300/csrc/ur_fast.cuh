@@ -9,7 +9,9 @@
 // ones; measured 22-23 % faster steps).
 #define UR_FAST_COL_E 16
 
-enum { P2_Y_FWD = 0, P2_Y_INV = 1, P2_Z_BIN = 2, P2_Z_ADJ = 3 };
+// P2_Y_INV_ROWS: P2_Y_INV that writes only the rows inside the particle (ColArgs::row_skip); the
+// launchers choose it, since the test costs the full inverse 6 % (512^3: 203 -> 215 us)
+enum { P2_Y_FWD = 0, P2_Y_INV = 1, P2_Z_BIN = 2, P2_Z_ADJ = 3, P2_Y_INV_ROWS = 4 };
 
 struct RowArgs {
   const void* ed;          // density rows (GEN = 0), plane-major, nrows x N
@@ -25,7 +27,7 @@ struct RowArgs {
   const float* weights;    // GEN >= 1 with UR_SHAPE_WEIGHTS: full-box weights
   const float2* tw;        // table exp(-2 pi i t / N), t < N
   const float2* stw;       // stage twiddles of the N/2-point transform (power-of-two kernels)
-  int skip_empty;          // GEN = 1, sphere, N <= 512: rows outside the particle are not written
+  int skip_empty;          // GEN >= 1: rows outside the particle (row_outside) are not written
 };
 
 struct GradArgs {

@@ -62,8 +62,30 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
   const int M = N >> 1, H = M + 1;
   const long long r0 = blk * RB;
   const FastDiv dm((uint32_t)M), dh((uint32_t)H);
-  // generated rows: row r = p N + y (r < 2^31) and the cell indices, by multiply-shift
-  const FastDiv dn((uint32_t)N), du((uint32_t)(GEN ? ra.ucell : 1));
+  // generated rows (r = p N + y < 2^31): what a row shares is formed once, by one thread per row
+  RowMask* rms = reinterpret_cast<RowMask*>(smem + (size_t)RB * M);
+  int* crow = reinterpret_cast<int*>(rms + RB);  // cell offset of the row; -1: past the last row
+  const FastDiv du((uint32_t)(GEN ? ra.ucell : 1));
+  if (GEN) {
+    const FastDiv dn((uint32_t)N);
+    bool some = false;
+    for (int t = threadIdx.x; t < RB; t += blockDim.x) {
+      const long long r = r0 + t;
+      if (r >= nrows) {
+        crow[t] = -1;
+        continue;
+      }
+      const int p = (int)dn.div((uint32_t)r), y = (int)r - p * N, z = ra.z0 + p;
+      RowMask rm;
+      rm.init(ra.sh, y, z);
+      rms[t] = rm;
+      crow[t] = (int)(du.mod((uint32_t)(z + ra.oz)) * ra.ucell + du.mod((uint32_t)(y + ra.oy)));
+      some = some || !rm.empty(ra.sh);
+    }
+    // rows outside the particle are not written when the y pass knows to skip them
+    const bool any = __syncthreads_or(some);
+    if (ra.skip_empty && !any) return;
+  }
   for (int f = threadIdx.x; f < RB * M; f += blockDim.x) {
     const int t = (int)dm.div((uint32_t)f);
     const int m = f - t * M;
@@ -71,24 +93,26 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
     float2 v = make_float2(0.f, 0.f);
     if (r < nrows) {
       if (GEN) {
-        const int p = (int)dn.div((uint32_t)r), y = (int)r - p * N, z = ra.z0 + p, x = 2 * m, U = ra.ucell;
-        const float* crow =
-            ra.cell + ((long long)du.mod((uint32_t)(z + ra.oz)) * U + du.mod((uint32_t)(y + ra.oy))) * U;
+        const int x = 2 * m, U = ra.ucell;
+        const int c0 = GEN == 2 ? 0 : (int)du.mod((uint32_t)(x + ra.ox));
+        const int c1 = c0 + 1 == U ? 0 : c0 + 1;
         float m0, m1;
         if (ra.weights) {
-          const float2 mw = __ldg(reinterpret_cast<const float2*>(ra.weights + ((long long)z * N + y) * N + x));
+          const float2 mw = __ldg(reinterpret_cast<const float2*>(ra.weights + ((long long)ra.z0 * N + r) * N + x));
           m0 = mw.x;
           m1 = mw.y;
         } else {
-          m0 = mask_at(ra.sh, x, y, z);
-          m1 = mask_at(ra.sh, x + 1, y, z);
+          m0 = rms[t].at(x);
+          m1 = rms[t].at(x + 1);
         }
-        if (GEN == 2)
+        if (GEN == 2) {
+          const int p = (int)(r / N), y = (int)(r - (long long)p * N), z = ra.z0 + p;
           v = make_float2(__fmul_rn(lattice_sample(ra.lat, ra.sh, ra.cell, U, x, y, z), m0),
                           __fmul_rn(lattice_sample(ra.lat, ra.sh, ra.cell, U, x + 1, y, z), m1));
-        else
-          v = make_float2(__fmul_rn(__ldg(crow + du.mod((uint32_t)(x + ra.ox))), m0),
-                          __fmul_rn(__ldg(crow + du.mod((uint32_t)(x + 1 + ra.ox))), m1));
+        } else {
+          const float* cr = ra.cell + (long long)crow[t] * U;
+          v = make_float2(__fmul_rn(__ldg(cr + c0), m0), __fmul_rn(__ldg(cr + c1), m1));
+        }
       } else {
         v = load_pair<T>(ed + r * N + 2 * m);
       }
@@ -131,65 +155,79 @@ struct ColDivs {
   __device__ explicit ColDivs(const ColArgs& a) : tx((uint32_t)a.TX), h((uint32_t)a.H) {}
 };
 
-__device__ __forceinline__ long long col_offset(uint32_t c, const FastDiv& dh, long long A) {
-  const uint32_t o = dh.div(c);
-  return (long long)o * A + (c - o * dh.d);
-}
+// Element access of the column transforms: element i of tile line `line` (column c0 + line) in the
+// source or destination layout, with the elements that are known to be zero or not needed left
+// out (ColArgs: row_skip, k2_zero, out_lo).
+// (Fields are copied: a batched launch holds its ColArgs in global memory.)
+template <int MODE, bool INV>
+struct ColLd {
+  const float2* src;
+  long long A, S, ncols, c0;
+  int zoff, nload, N, M, row_skip, gen_z0, k2_zero;
+  float cy, cz, rb2;
+  FastDiv h;
+  __device__ ColLd(const ColArgs& a, const ColDivs& dv, long long c)
+      : src(a.src), A(a.A), S(a.S), ncols(a.ncols), c0(c), zoff(a.zoff), nload(a.nload), N(a.N), M(a.M),
+        row_skip(a.row_skip), gen_z0(a.gen_z0), k2_zero(a.k2_zero), cy(a.sh.cy), cz(a.sh.cz), rb2(a.sh.rb2), h(dv.h) {}
+  __device__ __forceinline__ float2 operator()(int line, int i) const {
+    const long long c = c0 + line;
+    const int li = i - zoff;
+    if (c < ncols && li >= 0 && li < nload) {
+      const uint32_t o = h.div((uint32_t)c), k = (uint32_t)c - o * h.d;
+      if (MODE == COL_Y && !INV && row_skip && row_outside(cy, cz, rb2, i, gen_z0 + (int)o)) return make_float2(0.f, 0.f);
+      if (MODE == COL_Y && INV) {
+        const int ky = i < M ? i : i - N;
+        if ((int)(k * k) + ky * ky >= k2_zero) return make_float2(0.f, 0.f);
+      }
+      return __ldg(src + (long long)o * A + k + (long long)li * S);
+    }
+    return make_float2(0.f, 0.f);
+  }
+};
+template <int MODE, bool INV>
+struct ColSt {
+  float2* dst;
+  long long Ad, Sd, ncols, c0;
+  int row_skip, gen_z0, out_lo, out_cnt;
+  float cy, cz, rb2;
+  FastDiv h;
+  __device__ ColSt(const ColArgs& a, const ColDivs& dv, long long c)
+      : dst(a.dst), Ad(a.Ad), Sd(a.Sd), ncols(a.ncols), c0(c), row_skip(a.row_skip), gen_z0(a.gen_z0), out_lo(a.out_lo),
+        out_cnt(a.out_cnt), cy(a.sh.cy), cz(a.sh.cz), rb2(a.sh.rb2), h(dv.h) {}
+  __device__ __forceinline__ void operator()(int line, int i, float2 v) const {
+    const long long c = c0 + line;
+    if (c >= ncols) return;
+    const uint32_t o = h.div((uint32_t)c), k = (uint32_t)c - o * h.d;
+    if (MODE == COL_Y && INV && row_skip && row_outside(cy, cz, rb2, i, gen_z0 + (int)o)) return;
+    if (MODE == COL_ZADJ && out_cnt > 0) {
+      i -= out_lo;
+      if (i < 0 || i >= out_cnt) return;
+    }
+    dst[(long long)o * Ad + k + (long long)i * Sd] = v;
+  }
+};
 
-__device__ __forceinline__ void load_columns(const ColArgs& a, const ColDivs& dv, float2* buf, long long c0, int N) {
+// The tile's columns to shared memory and back, for transforms of a single stage
+template <class Ld>
+__device__ __forceinline__ void load_columns(const ColArgs& a, const ColDivs& dv, float2* buf, int N, Ld ld) {
   const int TX = a.TX;
   for (int f = threadIdx.x; f < TX * N; f += blockDim.x) {
     const int i = (int)dv.tx.div((uint32_t)f);
     const int t = f - i * TX;
-    const long long c = c0 + t;
-    const int li = i - a.zoff;
-    float2 v = make_float2(0.f, 0.f);
-    if (c < a.ncols && li >= 0 && li < a.nload) {
-      v = __ldg(a.src + col_offset((uint32_t)c, dv.h, a.A) + (long long)li * a.S);
-    }
-    buf[t * a.pitch + i] = v;
+    buf[t * a.pitch + i] = ld(t, i);
   }
   __syncthreads();
 }
 
-__device__ __forceinline__ void store_columns(const ColArgs& a, const ColDivs& dv, const float2* buf, long long c0,
-                                              int N) {
+template <class St>
+__device__ __forceinline__ void store_columns(const ColArgs& a, const ColDivs& dv, const float2* buf, int N, St st) {
   const int TX = a.TX;
   for (int f = threadIdx.x; f < TX * N; f += blockDim.x) {
     const int i = (int)dv.tx.div((uint32_t)f);
     const int t = f - i * TX;
-    const long long c = c0 + t;
-    if (c < a.ncols) a.dst[col_offset((uint32_t)c, dv.h, a.Ad) + (long long)i * a.Sd] = buf[t * a.pitch + i];
+    st(t, i, buf[t * a.pitch + i]);
   }
 }
-
-// Element access of the first and last transform stages (fft_lines_io): element i of
-// tile line `line` (column c0 + line) in the source or destination layout.
-struct ColLd {
-  const float2* src;
-  long long A, S, ncols, c0;
-  int zoff, nload;
-  FastDiv h;
-  __device__ ColLd(const ColArgs& a, const ColDivs& dv, long long c)
-      : src(a.src), A(a.A), S(a.S), ncols(a.ncols), c0(c), zoff(a.zoff), nload(a.nload), h(dv.h) {}
-  __device__ __forceinline__ float2 operator()(int line, int i) const {
-    const long long c = c0 + line;
-    const int li = i - zoff;
-    if (c < ncols && li >= 0 && li < nload) return __ldg(src + col_offset((uint32_t)c, h, A) + (long long)li * S);
-    return make_float2(0.f, 0.f);
-  }
-};
-struct ColSt {
-  float2* dst;
-  long long Ad, Sd, ncols, c0;
-  FastDiv h;
-  __device__ ColSt(const ColArgs& a, const ColDivs& dv, long long c)
-      : dst(a.dst), Ad(a.Ad), Sd(a.Sd), ncols(a.ncols), c0(c), h(dv.h) {}
-  __device__ __forceinline__ void operator()(int line, int i, float2 v) const {
-    const long long c = c0 + line;
-    if (c < ncols) dst[col_offset((uint32_t)c, h, Ad) + (long long)i * Sd] = v;
-  }
-};
 
 // Walk the (column, |kz|) pairs of the block's spectrum columns in chunks of
 // BIN_CHUNK consecutive |kz| = m.  k^2 = kx^2 + ky^2 + m^2 grows with m, so the
@@ -300,6 +338,26 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
   double* hs2 = nullptr;
   const long long c0 = blk * a.TX;
   const ColDivs dv(a);
+  if ((MODE == COL_ZBIN && a.nbins > 0 && !a.fout) || (MODE == COL_ZADJ && a.nbins > 0)) {
+    // a tile whose columns all lie at or beyond the closing threshold reaches no bin: nothing to bin,
+    // or zero output (left unwritten when the y pass reads it as zeros, k2_zero)
+    bool beyond = true;
+    for (int t = threadIdx.x; t < a.TX && c0 + t < a.ncols; t += blockDim.x) {
+      const uint32_t o = dv.h.div((uint32_t)(c0 + t));
+      const int kx = (int)((uint32_t)(c0 + t) - o * dv.h.d), ky = (int)o < a.M ? (int)o : (int)o - N;
+      beyond = beyond && kx * kx + ky * ky >= __ldg(a.thr + a.nbins);
+    }
+    if (__syncthreads_and(beyond)) {
+      if (MODE == COL_ZADJ && a.k2_zero == 0x7fffffff) {
+        const ColSt<MODE, INV> st(a, dv, c0);
+        for (int f = threadIdx.x; f < a.TX * N; f += blockDim.x) {
+          const int i = (int)dv.tx.div((uint32_t)f);
+          st(f - i * a.TX, i, make_float2(0.f, 0.f));
+        }
+      }
+      return;
+    }
+  }
   if (MODE != COL_Y && a.nbins > 0) {
     for (int j = threadIdx.x; j <= a.nbins; j += blockDim.x) thr[j] = __ldg(a.thr + j);
     if (MODE == COL_ZBIN) {
@@ -333,20 +391,21 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
     // with two or more stages the first stage reads the columns from global memory and, where
     // the result goes back to global memory, the last stage writes it (no staging round trips)
     const bool io = a.nst >= 2;
+    const ColLd<MODE, INV> ld(a, dv, c0);
+    const ColSt<MODE, INV> st(a, dv, c0);
     if (MODE == COL_Y) {
       if (io) {
-        fft_lines_io<INV, UR_EMAX, true, true, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ColLd(a, dv, c0),
-                                               ColSt(a, dv, c0));
+        fft_lines_io<INV, UR_EMAX, true, true, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ld, st);
       } else {
-        load_columns(a, dv, buf, c0, N);
+        load_columns(a, dv, buf, N, ld);
         fft_lines<INV, UR_EMAX>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw);
-        store_columns(a, dv, buf, c0, N);
+        store_columns(a, dv, buf, N, st);
       }
     } else if (MODE == COL_ZBIN) {
       if (io) {
-        fft_lines_io<false, UR_EMAX, true, false, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ColLd(a, dv, c0), NoSt());
+        fft_lines_io<false, UR_EMAX, true, false, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ld, NoSt());
       } else {
-        load_columns(a, dv, buf, c0, N);
+        load_columns(a, dv, buf, N, ld);
         fft_lines<false, UR_EMAX>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw);
       }
       if (a.fout) {
@@ -363,19 +422,19 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
       }
     } else {  // COL_ZADJ: F along z (recomputed or given), times sigma(bin), inverse along z
       if (io && !a.skip_fwd) {
-        fft_lines_io<false, UR_EMAX, true, false, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ColLd(a, dv, c0), NoSt());
+        fft_lines_io<false, UR_EMAX, true, false, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, ld, NoSt());
       } else {
-        load_columns(a, dv, buf, c0, N);
+        load_columns(a, dv, buf, N, ld);
         if (!a.skip_fwd) fft_lines<false, UR_EMAX>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw);
       }
       SigmaScale sc{buf, a.pitch, a.M, N, a.nbins, a.sigma};
       walk_bins(a, dv, thr, c0, sc);
       __syncthreads();
       if (io) {
-        fft_lines_io<true, UR_EMAX, false, true, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, NoLd(), ColSt(a, dv, c0));
+        fft_lines_io<true, UR_EMAX, false, true, true>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw, NoLd(), st);
       } else {
         fft_lines<true, UR_EMAX>(buf, a.pitch, a.TX, a.sched, a.nst, a.tw);
-        store_columns(a, dv, buf, c0, N);
+        store_columns(a, dv, buf, N, st);
       }
     }
   }
@@ -743,6 +802,9 @@ __global__ void __launch_bounds__(UR_BINQ_THREADS, 4) k_bin_half(const __grid_co
 // ---------------------------------------------------------------------------
 // Host: kernel configuration for a plan
 // ---------------------------------------------------------------------------
+// rows of a block, and per row its mask terms and cell offset
+size_t ur_row_smem(int rb, int M) { return (size_t)rb * (M * sizeof(float2) + sizeof(RowMask) + sizeof(int)); }
+
 size_t ur_colbin_smem(const ur_plan* p) {
   return ur_align_up((size_t)p->col_tx * (p->n + 1) * sizeof(float2), 16) + ur_align_up((size_t)(p->nbins + 1) * 4, 16) +
          (size_t)p->nbins * 16;
@@ -755,7 +817,7 @@ ur_status ur_configure_kernels(ur_plan* p) {
   p->row_rb = (UR_EMAX * p->row_threads) / M;
   if (p->row_rb > 64) p->row_rb = 64;
   if (p->row_rb < 1) p->row_rb = 1;
-  p->row_smem = (size_t)p->row_rb * M * sizeof(float2);
+  p->row_smem = ur_row_smem(p->row_rb, M);
   // columns: TX columns of N complex per block
   p->col_threads = 256;
   p->col_tx = (UR_EMAX * p->col_threads) / n;
@@ -865,9 +927,9 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
     r.nrows = np * n;
     r.z0 = ra.z0 + (int)p0;
     if (!gen) r.ed = (const char*)ra.ed + p0 * (long long)n * n * (p->ed_dtype == UR_F16 ? 2 : 4);
-    // generated sphere on rows of at most one warp: the row pass leaves the rows outside the
-    // particle unwritten and the y pass reads them as zeros
-    const bool skip = gen && p->fast && n <= 512 && ra.sh.kind == UR_SHAPE_SPHERE && !ra.weights;
+    // generated particle: the row pass leaves the rows outside it unwritten and the y pass reads them
+    // as zeros
+    const bool skip = gen && ra.sh.rb2 < INFINITY && !ra.weights;
     r.skip_empty = skip ? 1 : 0;
     ur_timing_begin("rows_r2c", s);
     if (p->fast) {

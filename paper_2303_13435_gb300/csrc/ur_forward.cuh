@@ -45,21 +45,25 @@ struct ColArgs {
   // adjoint
   const float* sigma;  // per-bin scale of F~ along z (adjoint)
   int skip_fwd;        // 1: the loaded column is already the spectrum along z
-  int row_skip;        // power-of-two forward y pass over a generated sphere density: rows
-  int gen_z0;          // (y, gen_z0 + plane) outside the sphere are zero and were not
-  ShapeArgs sh;        // written by the row pass; they are not read
+  int row_skip;        // rows (y, gen_z0 + plane) outside the particle (row_outside): forward y pass,
+  int gen_z0;          // they are zero, were not written by the row pass and are not read; adjoint
+  ShapeArgs sh;        // y pass, nobody reads them and they are not written
   int out_lo, out_cnt; // adjoint z pass: write only the planes z in [out_lo, out_lo + out_cnt), at
                        // z - out_lo (out_cnt = 0: every plane)
-  int k2_zero;         // power-of-two adjoint: spectrum columns with kx^2 + ky^2 >= k2_zero are
-                       // zero; the z pass may leave them unwritten and the y pass does not read
-                       // them (0x7fffffff: none)
+  int k2_zero;         // adjoint: spectrum columns with kx^2 + ky^2 >= k2_zero are zero; the z pass
+                       // may leave them unwritten and the y pass does not read them (0x7fffffff:
+                       // none)
 };
 
-// generic adjoint row pass (one block: a batch of rows wrapping onto one cell row)
+// generic adjoint row pass (one block: up to RB rows wrapping onto G neighbouring cell rows)
 struct GenGradArgs {
   const float2* Y;
   int yp;            // row pitch of Y
   int N, RB, nst;
+  int zlo, zhi;      // planes to process; Y starts at plane zlo
+  int ylo, yhi;      // rows to process
+  int G, nza, nyb;   // cell rows per block; row slots per cell row: nza planes x nyb rows
+  int row_skip;      // 1: rows outside the particle are not needed
   const StageInfo* sched;
   const float2* tw;
   const float* cell;
@@ -109,6 +113,16 @@ ur_status ur_batch_launch_zero(const BatchZeroItem* items, int count, cudaStream
 ur_status ur_batch_launch_grad(const BatchGradItem* items, const long long* start, int count, long long nblocks,
                                size_t smem, cudaStream_t s);
 
+// What an adjoint has to produce: planes [zlo, zhi) and rows [ylo, yhi) of dL/drho.  All of them for
+// dL/dm; for dL/du alone only those that the mask can reach (row_skip: nor rows outside it).
+struct AdjRange {
+  int zlo, zhi, ylo, yhi, row_skip;
+};
+AdjRange ur_adj_range(const ur_plan* p, const ShapeArgs& sh, bool want_mask);
+int ur_k2_zero(const ur_plan* p);
+void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy);
+size_t ur_grad_smem(const ur_plan* p);
+size_t ur_row_smem(int rb, int M);
 ColArgs ur_col_args(const ur_plan* p);
 ur_status ur_plane_pass(const ur_plan* p, const void* ed, long long nplanes, float2* X, cudaStream_t s);
 ur_status ur_column_pass(const ur_plan* p, const float2* X, double* bins, float2* F_out, cudaStream_t s);

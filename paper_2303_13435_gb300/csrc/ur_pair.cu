@@ -104,7 +104,7 @@ template <int N, int MODE>
 struct PairCfg {
   static constexpr int E = 8, LE = 3;
   static constexpr int T = N / E;
-  static constexpr int THREADS = N == 512 && (MODE == P2_Y_INV || MODE == P2_Z_ADJ) ? 512 : 256;
+  static constexpr int THREADS = N == 512 && (MODE == P2_Y_INV || MODE == P2_Y_INV_ROWS || MODE == P2_Z_ADJ) ? 512 : 256;
   static constexpr int TXP = THREADS / T;
   static constexpr int MINB = 1024 / THREADS;
   // column pitch in 16-byte words: the eight lanes of a phase are TXP columns of 8 / TXP positions
@@ -183,7 +183,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::MINB)) k_pair_cols(const __grid_constant__ ColArgs a) {
   using Cfg = PairCfg<N, MODE>;
   constexpr int E = Cfg::E, T = Cfg::T, TXP = Cfg::TXP, PITCH = Cfg::PITCH, CW = Cfg::CW, M = N / 2, H = M + 1;
-  constexpr bool ZP = MODE == P2_Z_BIN || MODE == P2_Z_ADJ;
+  constexpr bool ZP = MODE == P2_Z_BIN || MODE == P2_Z_ADJ, YINV = MODE == P2_Y_INV || MODE == P2_Y_INV_ROWS;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_blo, s_bhi;
   ulonglong2* buf = reinterpret_cast<ulonglong2*>(smraw);
@@ -259,9 +259,9 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
         la = la && in;
         lb = lb && in;
       } else if (MODE == P2_Y_FWD) {
-        if (a.row_skip) {  // rows outside a generated sphere were not written
-          la = la && !sphere_row_empty(a.sh, li, a.gen_z0 + ia);
-          lb = lb && !sphere_row_empty(a.sh, li, a.gen_z0 + ib);
+        if (a.row_skip) {  // rows outside the particle were not written
+          la = la && !row_outside(a.sh, li, a.gen_z0 + ia);
+          lb = lb && !row_outside(a.sh, li, a.gen_z0 + ib);
         }
       } else {  // columns at or beyond k2_zero were not written
         const int ky = li < M ? li : li - N;
@@ -284,8 +284,16 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
     atomicMax(&s_bhi, hi_bin);
   }
   if (!ZP) {
-    pair_stages<N, MODE == P2_Y_INV, 0>(v, j, line, tw);
-    if (valid) {
+    pair_stages<N, YINV, 0>(v, j, line, tw);
+    if (MODE == P2_Y_INV_ROWS) {  // rows outside the particle are not needed
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const float2 x = f2_get(v[q].x), y = f2_get(v[q].y);
+        const int li = j + q * T;
+        if (valid && !row_outside(a.sh, li, a.gen_z0 + ia)) *at_step(da + j * a.Sd, q, dstep) = make_float2(x.x, y.x);
+        if (hasb && !row_outside(a.sh, li, a.gen_z0 + ib)) *at_step(db + j * a.Sd, q, dstep) = make_float2(x.y, y.y);
+      }
+    } else if (valid) {
 #pragma unroll
       for (int q = 0; q < E; ++q)
         c2_store(at_step(da + j * a.Sd, q, dstep), at_step(db + j * a.Sd, q, dstep), hasb, v[q]);
@@ -457,7 +465,7 @@ template <int N>
 static ur_status launch_pair_n(int mode, const ColArgs& a, cudaStream_t s) {
   switch (mode) {
     case P2_Y_FWD: return launch_pair<N, P2_Y_FWD>(a, s);
-    case P2_Y_INV: return launch_pair<N, P2_Y_INV>(a, s);
+    case P2_Y_INV: return a.row_skip ? launch_pair<N, P2_Y_INV_ROWS>(a, s) : launch_pair<N, P2_Y_INV>(a, s);
     case P2_Z_BIN: return launch_pair<N, P2_Z_BIN>(a, s);
     default: return launch_pair<N, P2_Z_ADJ>(a, s);
   }
