@@ -153,9 +153,20 @@ __device__ __forceinline__ float2 ld_pair<__half>(const __half* p) {
   return __half22float2(__ldg(reinterpret_cast<const __half2*>(p)));
 }
 
+// Values per thread: 8, and 16 for stored rows of N = 1024, where a row then is one warp as it is below
+// (warp barriers only): 1024^3 FP16 rows 2270 -> 1849 us, FP16 slabs of the streamed forward 302 -> 174 us.
+// Generated rows (541 -> 597 us) and the adjoint rows (2612 -> 3056 us) at 1024, with 64 and 80 registers,
+// and two and more warps per row (2048 on: 1-3 %) were slower with 16.
+template <int N, int GEN>
+struct RowCfg {
+  static constexpr int E = GEN == 0 ? UR_FAST_STORED_ROW_E(N) : 8;
+  static constexpr int THREADS = E == 16 ? 256 : 512;
+};
+
 template <int N, int GEN, typename TED>
-__global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
-  constexpr int M = N / 2, H = M + 1, T = M / 8, RB = 512 / T, PITCH = P2<M>::PITCH;
+__global__ void __launch_bounds__((RowCfg<N, GEN>::THREADS), (RowCfg<N, GEN>::E == 16 ? 4 : 3)) k_p2_rows(RowArgs a) {
+  constexpr int E = RowCfg<N, GEN>::E, M = N / 2, H = M + 1, T = M / E, RB = RowCfg<N, GEN>::THREADS / T;
+  constexpr int PITCH = P2<M, E>::PITCH;
   // a row of up to 256 complex values is one warp (or part of one): warp barriers only
   constexpr bool WS = T <= 32;
   __shared__ __align__(16) float2 sm[RB * PITCH];
@@ -164,9 +175,9 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
   const bool valid = r < a.nrows;
   const unsigned wmask = p2_line_lanes<T>();
   float2* line = sm + t * PITCH;
-  float2 v[8];
+  float2 v[E];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = make_float2(0.f, 0.f);
+  for (int q = 0; q < E; ++q) v[q] = make_float2(0.f, 0.f);
   if (GEN) {
     const int p = (int)(r / N), y = (int)(r - (long long)p * N);
     const int z = a.z0 + p;
@@ -187,7 +198,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
       rm.init(a.sh, y, z);
       if constexpr (GEN == 2) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < E; ++q) {
           const int x = 2 * (j + q * T);
           float m0, m1;
           if (wrow) {
@@ -208,7 +219,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
         const int cstep = a.fu.mod(2 * T);
         int c0 = a.fu.mod(2 * j + a.ox);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < E; ++q) {
           const int x = 2 * (j + q * T);
           float m0, m1;
           if (wrow) {
@@ -229,27 +240,27 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
   } else if (valid) {
     const TED* row = reinterpret_cast<const TED*>(a.ed) + r * N;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = ld_pair<TED>(row + 2 * (j + q * T));
+    for (int q = 0; q < E; ++q) v[q] = ld_pair<TED>(row + 2 * (j + q * T));
   }
   // a row whose values are all zero transforms to zero: skip its butterflies
   bool zero_row = false;
   if constexpr (WS) {
     bool nz = false;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) nz |= (v[q].x != 0.f) || (v[q].y != 0.f);
+    for (int q = 0; q < E; ++q) nz |= (v[q].x != 0.f) || (v[q].y != 0.f);
     zero_row = (__ballot_sync(wmask, nz) & wmask) == 0u;
   }
-  if (!zero_row) p2_fft<M, false, WS>(v, j, line, a.stw, wmask);
+  if (!zero_row) p2_fft<M, false, WS, E>(v, j, line, a.stw, wmask);
   // split step: X[k] = (Z[k] + conj Z[M-k])/2 - i W_N^k (Z[k] - conj Z[M-k])/2
   if constexpr (WS) {
-    // Z[M - k], k = j + qT, is register 7 - q of lane T - j of the same row (j >= 1);
-    // lane j = 0 holds its own partners: Z[M - qT] = its register 8 - q, and Z[0]
+    // Z[M - k], k = j + qT, is register E - 1 - q of lane T - j of the same row (j >= 1);
+    // lane j = 0 holds its own partners: Z[M - qT] = its register E - q, and Z[0]
     const int src = ((threadIdx.x & 31) & ~(T - 1)) | ((T - j) & (T - 1));
     float2* X = a.X + (valid ? r : 0) * a.xp;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      float2 zm = make_float2(__shfl_sync(wmask, v[7 - q].x, src), __shfl_sync(wmask, v[7 - q].y, src));
-      if (j == 0) zm = v[(8 - q) & 7];
+    for (int q = 0; q < E; ++q) {
+      float2 zm = make_float2(__shfl_sync(wmask, v[E - 1 - q].x, src), __shfl_sync(wmask, v[E - 1 - q].y, src));
+      if (j == 0) zm = v[(E - q) & (E - 1)];
       if (!valid) continue;
       const int k = j + q * T;
       if (zero_row) {
@@ -272,15 +283,15 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows(RowArgs a) {
   }
   if (!zero_row) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) line[p2pad(j + q * T)] = v[q];
+    for (int q = 0; q < E; ++q) line[p2pad(j + q * T)] = v[q];
   }
   p2_sync<WS>(wmask);
   if (valid) {
     float2* X = a.X + r * a.xp;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
+    for (int q = 0; q < E + 1; ++q) {
       int k = j + q * T;
-      if (q == 8) {
+      if (q == E) {
         if (j != 0) break;
         k = M;
       }
@@ -582,7 +593,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
 // CELL: dL/du alone; rows that the mask excludes entirely add nothing to it and are left out.
 template <int N, bool CELL>
 __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
-  constexpr int M = N / 2, H = M + 1, T = M / 8, PITCH = P2<M>::PITCH + 1;
+  constexpr int E = 8, M = N / 2, H = M + 1, T = M / E, PITCH = P2<M, E>::PITCH + 1;
   constexpr bool WS = T <= 32;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int RB = a.rb;
@@ -606,21 +617,21 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
   for (int i = threadIdx.x; i < U; i += blockDim.x) acc[i] = 0.f;
   float2* line = sm + t * PITCH;
   const float2* Yrow = a.Y + ((long long)(z - a.ybase_z) * N + (valid ? y : 0)) * a.yp;
-  // all nine loads of the row (k = j + q T, and k = M) are issued together
-  float2 ld[9];
+  // all E + 1 loads of the row (k = j + q T, and k = M) are issued together
+  float2 ld[E + 1];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) ld[q] = live ? __ldg(Yrow + j + q * T) : make_float2(0.f, 0.f);
-  ld[8] = (live && j == 0) ? __ldg(Yrow + M) : make_float2(0.f, 0.f);
-  float2 v[8];
+  for (int q = 0; q < E; ++q) ld[q] = live ? __ldg(Yrow + j + q * T) : make_float2(0.f, 0.f);
+  ld[E] = (live && j == 0) ? __ldg(Yrow + M) : make_float2(0.f, 0.f);
+  float2 v[E];
   if constexpr (WS) {
-    // X[M - k], k = j + qT, is load 7 - q of lane T - j of the same row (j >= 1); lane
-    // j = 0 holds its own partners: X[M - qT] = its load 8 - q (X[M] for q = 0)
+    // X[M - k], k = j + qT, is load E - 1 - q of lane T - j of the same row (j >= 1); lane
+    // j = 0 holds its own partners: X[M - qT] = its load E - q (X[M] for q = 0)
     const int src = ((threadIdx.x & 31) & ~(T - 1)) | ((T - j) & (T - 1));
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < E; ++q) {
       const int k = j + q * T;
-      float2 xb = make_float2(__shfl_sync(wmask, ld[7 - q].x, src), __shfl_sync(wmask, ld[7 - q].y, src));
-      if (j == 0) xb = ld[8 - q];
+      float2 xb = make_float2(__shfl_sync(wmask, ld[E - 1 - q].x, src), __shfl_sync(wmask, ld[E - 1 - q].y, src));
+      if (j == 0) xb = ld[E - q];
       const float2 xa = ld[q];
       const float2 w = __ldg(a.tw + k);
       const float2 e = cadd(xa, cconj(xb));
@@ -631,11 +642,11 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
     __syncthreads();  // orders the zeroing of acc before any accumulation
   } else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) line[p2pad(j + q * T)] = ld[q];
-    if (j == 0) line[p2pad(M)] = ld[8];
+    for (int q = 0; q < E; ++q) line[p2pad(j + q * T)] = ld[q];
+    if (j == 0) line[p2pad(M)] = ld[E];
     __syncthreads();  // also orders the zeroing of acc before any accumulation
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < E; ++q) {
       const int k = j + q * T;
       const float2 xa = line[p2pad(k)], xb = line[p2pad(M - k)];
       const float2 w = __ldg(a.tw + k);
@@ -646,7 +657,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
     }
     __syncthreads();  // the transform's first exchange reuses the lines
   }
-  if (!CELL || !WS || live) p2_fft<M, true, WS>(v, j, line, a.stw, wmask);
+  if (!CELL || !WS || live) p2_fft<M, true, WS, E>(v, j, line, a.stw, wmask);
   const float* crow = a.cell + ((long long)cz * U + cy) * U;
   RowMask rm;
   rm.init(a.sh, valid ? y : 0, z);
@@ -665,7 +676,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
       const float u0 = __ldg(crow + c0), u1 = __ldg(crow + c1);
       float r0 = 0.f, r1 = 0.f;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < E; ++q) {
         const int x = 2 * (j + q * T);
         const float g0 = v[q].x * a.inv_n3, g1 = v[q].y * a.inv_n3;
         if (drow) *reinterpret_cast<float2*>(drow + x) = make_float2(g0 * u0, g1 * u1);
@@ -687,7 +698,7 @@ __global__ void __launch_bounds__(512, 3) k_p2_rows_grad(GradArgs a) {
       if (r1 != 0.f) atomicAdd(acc + c1, r1);
     } else {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
+      for (int q = 0; q < E; ++q) {
         const int x = 2 * (j + q * T);
         const float g0 = v[q].x * a.inv_n3, g1 = v[q].y * a.inv_n3;
         const int c1 = c0 + 1 == U ? 0 : c0 + 1;
@@ -766,15 +777,20 @@ ur_status ur_fast_cols(int n, int mode, const ColArgs& a, cudaStream_t s) {
   return UR_ERR_UNSUPPORTED;
 }
 
+template <int N, int GEN, typename TED>
+static void launch_rows(const RowArgs& a, cudaStream_t s) {
+  using Cfg = RowCfg<N, GEN>;
+  constexpr int RB = Cfg::THREADS / (N / 2 / Cfg::E);
+  k_p2_rows<N, GEN, TED><<<(unsigned)((a.nrows + RB - 1) / RB), Cfg::THREADS, 0, s>>>(a);
+}
+
 template <int N>
 static ur_status launch_rows_n(const RowArgs& a, int gen, int ed_f16, cudaStream_t s) {
-  constexpr int M = N / 2, T = M / 8, RB = 512 / T;
-  const int grid = (int)((a.nrows + RB - 1) / RB);
-  if (grid <= 0) return UR_OK;
-  if (gen == 2) k_p2_rows<N, 2, float><<<grid, 512, 0, s>>>(a);
-  else if (gen) k_p2_rows<N, 1, float><<<grid, 512, 0, s>>>(a);
-  else if (ed_f16) k_p2_rows<N, 0, __half><<<grid, 512, 0, s>>>(a);
-  else k_p2_rows<N, 0, float><<<grid, 512, 0, s>>>(a);
+  if (a.nrows <= 0) return UR_OK;
+  if (gen == 2) launch_rows<N, 2, float>(a, s);
+  else if (gen) launch_rows<N, 1, float>(a, s);
+  else if (ed_f16) launch_rows<N, 0, __half>(a, s);
+  else launch_rows<N, 0, float>(a, s);
   UR_LAUNCH_CHECK("k_p2_rows");
   return UR_OK;
 }

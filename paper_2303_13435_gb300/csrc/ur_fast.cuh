@@ -8,6 +8,8 @@
 // 16 from 1024 on (single columns, ur_fast.cu: three radix-16 stages at 4096 instead of four radix-8
 // ones; measured 22-23 % faster steps).
 #define UR_FAST_COL_E 16
+// ... and of the transforms of stored rows of n reals (generated rows and the adjoint rows: 8)
+#define UR_FAST_STORED_ROW_E(n) ((n) == 1024 ? 16 : 8)
 
 // P2_Y_INV_ROWS: P2_Y_INV that writes only the rows inside the particle (ColArgs::row_skip); the
 // launchers choose it, since the test costs the full inverse 6 % (512^3: 203 -> 215 us)

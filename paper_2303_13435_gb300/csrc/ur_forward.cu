@@ -920,7 +920,7 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
   for (long long p0 = 0; p0 < nplanes; p0 += step) {
     const long long np = (p0 + step <= nplanes) ? step : nplanes - p0;
     RowArgs r = ra;
-    r.stw = p->stw ? p->stw + p->stw_m_off : nullptr;
+    r.stw = p->stw ? p->stw + (gen ? p->stw_m_off : p->stw_s_off) : nullptr;
     r.fu = FastDiv((uint32_t)(ra.ucell > 0 ? ra.ucell : 1));
     r.X = X + p0 * n * p->xp;
     r.xp = p->xp;

@@ -426,17 +426,20 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
     int lg = 0;
     while ((1 << lg) < n) ++lg;
     // columns (N points): the pair table, or stages of UR_FAST_COL_E values per thread; rows (N/2
-    // points) 8
+    // points) 8, stored rows UR_FAST_STORED_ROW_E(n)
     const bool pair = ur_pair_supported(n);
     const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : stage_twiddles(lg, UR_FAST_COL_E, nullptr);
-    const size_t cm = stage_twiddles(lg - 1, 8, nullptr);
-    float2* st_h = (float2*)malloc(sizeof(float2) * (cn + cm + 1));
+    const int erow = UR_FAST_STORED_ROW_E(n);
+    const size_t cm = stage_twiddles(lg - 1, 8, nullptr), cs = erow == 8 ? 0 : stage_twiddles(lg - 1, erow, nullptr);
+    float2* st_h = (float2*)malloc(sizeof(float2) * (cn + cm + cs + 1));
     if (pair) ur_pair_twiddles(n, (float4*)st_h);
     else stage_twiddles(lg, UR_FAST_COL_E, st_h);
     stage_twiddles(lg - 1, 8, st_h + cn);
     p->stw_m_off = (int)cn;
-    const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (cn + cm + 1));
-    const cudaError_t eb = ea == cudaSuccess ? cudaMemcpy(p->stw, st_h, sizeof(float2) * (cn + cm + 1),
+    p->stw_s_off = cs ? (int)(cn + cm) : p->stw_m_off;
+    if (cs) stage_twiddles(lg - 1, erow, st_h + cn + cm);
+    const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (cn + cm + cs + 1));
+    const cudaError_t eb = ea == cudaSuccess ? cudaMemcpy(p->stw, st_h, sizeof(float2) * (cn + cm + cs + 1),
                                                           cudaMemcpyHostToDevice) : ea;
     free(st_h);
     if (eb != cudaSuccess) {
