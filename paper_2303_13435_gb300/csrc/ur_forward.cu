@@ -21,7 +21,10 @@
 
 #include "ur_fast.cuh"
 
-#define BIN_CHUNK 8  // consecutive |kz| per thread in the binning walk
+// Consecutive |kz| per thread in the binning and scaling walks; lanes read BIN_CHUNK values apart in
+// shared memory, so an odd number spreads them over the banks (8 -> 9: 378^3 z + bins 253 -> 245 us, adjoint
+// z 285 -> 268; 64 particles 3627 -> 3461 and 4374 -> 4059; 7 and 11 within 3 % of 9)
+#define BIN_CHUNK 9
 
 // ---------------------------------------------------------------------------
 // Pass 1a
