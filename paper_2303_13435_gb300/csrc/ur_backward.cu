@@ -43,7 +43,10 @@ __global__ void k_sigma(const double* __restrict__ g, const double* __restrict__
 // compare-and-swap loop.  64 particles of 96^3-384^3, dL/du only: 8674 -> 678 us (64-row tiles of
 // which 1 to 36 rows were used, every row of the box); 378^3 with dL/dm: 311 -> 289 us.
 struct NoStore {
-  __device__ __forceinline__ void operator()(int, int, float2) const {}
+  struct It {
+    __device__ __forceinline__ void put(float2) {}
+  };
+  __device__ __forceinline__ It first(int, int, int) const { return {}; }
 };
 
 struct GradRow {
@@ -129,7 +132,7 @@ __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int
       const float2 o = make_float2(d.x * w.x + d.y * w.y, d.y * w.x - d.x * w.y);  // * conj(W^i)
       return make_float2(e.x - o.y, e.y + o.x);
     };
-    fft_lines_io<true, UR_EMAX, true, false, false>(buf, H, nrow, sched, nst, tw, packed, NoStore());
+    fft_lines_io<true, UR_EMAX, true, false, false>(buf, H, nrow, sched, nst, tw, ld_fn(packed), NoStore());
   } else {
     for (int f = threadIdx.x; f < nrow * H; f += blockDim.x) {
       const int t = (int)dH.div((uint32_t)f);

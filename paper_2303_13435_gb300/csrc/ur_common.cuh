@@ -482,9 +482,29 @@ __device__ __forceinline__ void fft_lines(float2* buf, int pitch, int lines, con
   i = fft_stages_of<7, INV, EMAX>(buf, pitch, lines, s_st, nst, tw, i);
 }
 
-// First stage (Ns = 1, no twiddles) with inputs from `ld(line, i)` instead of shared
-// memory, and last stage (k = j, outputs at j + r Ns) handing its outputs to
-// `st(line, i, v)`.  Their butterflies are mapped line-fastest (w = j lines + line), so
+// Elements of a first stage from a function of (line, i)
+template <class F>
+struct LdFn {
+  F f;
+  struct It {
+    const F& f;
+    int line, i, di;
+    __device__ __forceinline__ float2 get() {
+      const float2 v = f(line, i);
+      i += di;
+      return v;
+    }
+  };
+  __device__ __forceinline__ It first(int line, int i, int di) const { return {f, line, i, di}; }
+};
+template <class F>
+__device__ __forceinline__ LdFn<F> ld_fn(const F& f) {
+  return {f};
+}
+
+// First stage (Ns = 1, no twiddles) with inputs from `ld` instead of shared memory, and
+// last stage (k = j, outputs at j + r Ns) handing its outputs to `st`: ld.first(line, i, di)
+// gives the elements i, i + di, ... of a line one after the other, st.first takes them.  Their butterflies are mapped line-fastest (w = j lines + line), so
 // consecutive threads take the same position of consecutive lines: a tile of columns is
 // read and written in row segments.
 template <int R, bool INV, int EMAX, bool LF, class Ld>
@@ -506,8 +526,9 @@ __device__ __forceinline__ void fft_first_stage(float2* __restrict__ buf, int pi
         j = w - line * nb;
       }
       float2 v[R];
+      auto in = ld.first(line, j, nb);
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = ld(line, j + r * nb);
+      for (int r = 0; r < R; ++r) v[r] = in.get();
       dft<R, INV>(v);
       float2* dst = buf + line * pitch + j * R;
 #pragma unroll
@@ -546,8 +567,9 @@ __device__ __forceinline__ void fft_last_stage(const float2* __restrict__ buf, i
         for (int r = 1; r < R; ++r) v[r] = twmul<INV>(v[r], ld_twiddle(tw + r * step));
       }
       dft<R, INV>(v);
+      auto out = st.first(line, j, nb);
 #pragma unroll
-      for (int r = 0; r < R; ++r) st(line, j + r * nb, v[r]);
+      for (int r = 0; r < R; ++r) out.put(v[r]);
     }
   }
 }
