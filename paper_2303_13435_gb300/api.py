@@ -158,7 +158,8 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the raw handle of the current stream, without building a torch.cuda.Stream around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
@@ -175,16 +176,9 @@ def _torch_dtype(code: int):
 
 
 def shape_desc(shape) -> ShapeDesc:
-    d = ShapeDesc()
-    d.kind = int(shape.kind)
-    c = np.asarray(shape.center, dtype=np.float32)
-    for i in range(3):
-        d.center[i] = float(c[i])
-    d.size = float(np.float32(shape.size))
-    r = np.asarray(shape.rot, dtype=np.float32).reshape(9)
-    for i in range(9):
-        d.rot[i] = float(r[i])
-    return d
+    c = np.asarray(shape.center, dtype=np.float32).tolist()
+    r = np.asarray(shape.rot, dtype=np.float32).reshape(9).tolist()
+    return ShapeDesc(int(shape.kind), (C.c_float * 3)(*c), float(np.float32(shape.size)), (C.c_float * 9)(*r))
 
 
 class Plan:

@@ -32,14 +32,14 @@ class UltimaRatioIQ(torch.autograd.Function):
         bins = api.fft_intensity_tiled(plan, cell, shape, origin=origin, weights=weights, ws=ws)
         ctx.plan, ctx.shape, ctx.origin, ctx.gen = plan, shape, origin, gen
         ctx.has_weights = weights is not None
-        ctx.save_for_backward(cell, weights if weights is not None else torch.empty(0, device=cell.device), bins)
+        ctx.save_for_backward(cell, weights, bins)
         return bins[api.BIN_MEAN].clone()
 
     @staticmethod
     def backward(ctx, g_mean):
         cell, weights, bins = ctx.saved_tensors
-        weights = weights if ctx.has_weights else None
-        g = torch.where(bins[api.BIN_COUNT] > 0, torch.nan_to_num(g_mean.to(torch.float64)), 0.0).contiguous()
+        # (empty bins, whose mean is NaN, get a zero scale in ur_backward whatever their gradient is)
+        g = torch.nan_to_num(g_mean.to(torch.float64)).contiguous()
         want_mask = ctx.has_weights and ctx.needs_input_grad[1]
         plan = ctx.plan
         if plan.workspace_generation() != ctx.gen:
