@@ -737,6 +737,7 @@ struct ur_plan {
   float2* tw;        // device [n]
   float2* stw;       // power-of-two path: stage twiddles of the N-point and (at stw_m_off) the N/2-point transforms
   int stw_m_off;
+  int stw_32_off;    // N-point transform with 32 values per thread
   int stw_s_off;     // N/2-point transform of stored rows
   int32_t* thr;      // device [nbins+1]
   int16_t* binlut;     // device [3 (N/2)^2 + 1]: bin of k^2 = s, -1 outside every bin

@@ -1,13 +1,13 @@
 // Power-of-two grid edges (64 <= N <= 4096): compile-time transforms.
 //
-// A length-L line is held by L/8 threads, eight complex values each
-// (thread j holds positions j + q L/8, q = 0..7).  Each Stockham stage is a
-// radix-8 butterfly in registers (the last stage radix 4 or 2 when log2 L is
-// not a multiple of 3); between stages the values cross shared memory once,
-// at padded addresses i + i/16 so that neither the strided writes nor the
-// contiguous reads conflict in banks.  After the last stage a thread again
-// holds positions j + q L/8, so the first stage can read and the last stage
-// can write global memory directly.
+// A length-L line is held by L/E threads, E = 8, 16 or 32 complex values each
+// (thread j holds positions j + q L/E, q < E).  Each Stockham stage is a radix-E
+// butterfly in registers (the last stage of a smaller radix when log2 L is not a
+// multiple of log2 E); between stages the values cross shared memory once,
+// at padded addresses so that neither the strided writes nor the contiguous
+// reads conflict in banks.  After the last stage a thread again holds
+// positions j + q L/E, so the first stage can read and the last stage can write
+// global memory directly.
 //
 // Kernels (Sec. 2.4 Eq. 2 split, Sec. 2.5 binning, and the adjoint):
 //   k_p2_rows<N, GEN>  rows along x: real-to-complex via an N/2-point
@@ -23,24 +23,24 @@
 #include "ur_density.cuh"
 #include "ur_fast.cuh"
 
-// E = values per thread: 8 (radix-8 stages) or 16 (radix-16 stages, used by the
-// column passes of the longest lines, where fewer exchanges per transform and
-// more values per barrier pay for the registers).
+// E = values per thread: 8, 16 or 32 (the column passes of the longer lines, where fewer
+// exchanges per transform and more values per barrier pay for the registers).
 template <int L, int E = 8>
 struct P2 {
   static constexpr int LOG = L == 8 ? 3 : L == 16 ? 4 : L == 32 ? 5 : L == 64 ? 6 : L == 128 ? 7 : L == 256 ? 8
                                                                                            : L == 512 ? 9 : L == 1024 ? 10
                                                                                            : L == 2048 ? 11 : 12;
-  static constexpr int LE = E == 16 ? 4 : 3;  // log2 E
+  static constexpr int LE = E == 32 ? 5 : E == 16 ? 4 : 3;  // log2 E
   static constexpr int T = L / E;
   static constexpr int NFULL = LOG / LE;
   static constexpr int REM = LOG % LE;
   static constexpr int NST = NFULL + (REM ? 1 : 0);
-  static constexpr int PITCH = L + L / 16;
-  static_assert(E == 8 || E == 16, "8 or 16 values per thread");
+  static constexpr int PITCH = L + L / (E == 32 ? 32 : 16);
+  static_assert(E == 8 || E == 16 || E == 32, "8, 16 or 32 values per thread");
 };
 
-__device__ __forceinline__ int p2pad(int i) { return i + (i >> 4); }
+template <int E = 8>
+__device__ __forceinline__ int p2pad(int i) { return i + (i >> (E == 32 ? 5 : 4)); }
 
 constexpr int ipowe(int e, int s) { return s == 0 ? 1 : e * ipowe(e, s - 1); }
 
@@ -106,11 +106,11 @@ __device__ __forceinline__ void p2_exchange(float2 (&v)[E], int j, float2* line,
     const int b = j + i * T;
     const int k = b & (NS - 1);
 #pragma unroll
-    for (int r = 0; r < R; ++r) line[p2pad((b - k) * R + k + r * NS)] = v[i + NB * r];
+    for (int r = 0; r < R; ++r) line[p2pad<E>((b - k) * R + k + r * NS)] = v[i + NB * r];
   }
   p2_sync<WS>(wmask);
 #pragma unroll
-  for (int q = 0; q < E; ++q) v[q] = line[p2pad(j + q * T)];
+  for (int q = 0; q < E; ++q) v[q] = line[p2pad<E>(j + q * T)];
   p2_sync<WS>(wmask);
 }
 
@@ -313,21 +313,25 @@ __global__ void __launch_bounds__((RowCfg<N, GEN>::THREADS), (RowCfg<N, GEN>::E 
 // Columns.  Block = TX columns x L/E threads; thread (j, c), c fastest, so a
 // warp reads whole row segments of TX consecutive columns.
 // ---------------------------------------------------------------------------
-// Threads per column block: 512, or 1024 for N >= 2048 so that a block still spans at least two
-// columns (16-byte row segments) of the half spectrum; 16 values per thread take 64 registers.
-template <int N>
+// Values per thread and threads per block.  At 1024 the passes without binning hold 32 values per thread
+// (1024 = 32 32: one shared-memory exchange instead of two; 128 registers, two blocks of 256 threads): y 823 ->
+// 719 us, adjoint z 2540 -> 2475, adjoint y 1955 -> 1691; the binned pass keeps 16 (2200 -> 2461 us with 32: a
+// walk twice as long per thread).  512 points gain nothing by it (91 -> 113 us against pairs).  16 values per
+// thread take 64 registers and blocks of 512 threads, or 1024 for N >= 2048 so that a block still spans
+// at least two columns (16-byte row segments) of the half spectrum.
+template <int N, int MODE>
 struct ColCfg {
-  static constexpr int E = UR_FAST_COL_E;
-  static constexpr int THREADS = N >= 2048 ? 1024 : 512;
+  static constexpr int E = UR_FAST_COL_E(N, MODE);
+  static constexpr int THREADS = N >= 2048 ? 1024 : E == 32 ? 256 : 512;
   static constexpr int TX = THREADS / (N / E);
-  static constexpr int MINB = 65536 / (64 * THREADS);
+  static constexpr int MINB = E == 32 ? 2 : 65536 / (64 * THREADS);
 };
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols(ColArgs a) {
+__global__ void __launch_bounds__((ColCfg<N, MODE>::THREADS), (ColCfg<N, MODE>::MINB)) k_p2_cols(ColArgs a) {
   // column pitch = 2 (mod 16) float2: the TX columns a warp touches fall on different banks
-  constexpr int E = ColCfg<N>::E;
-  constexpr int T = N / E, TX = ColCfg<N>::TX, PITCH = P2<N>::PITCH + 2, H = N / 2 + 1, M = N / 2;
+  constexpr int E = ColCfg<N, MODE>::E;
+  constexpr int T = N / E, TX = ColCfg<N, MODE>::TX, PITCH = P2<N, E>::PITCH + 2, H = N / 2 + 1, M = N / 2;
   constexpr bool YINV = MODE == P2_Y_INV || MODE == P2_Y_INV_ROWS;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_blo, s_bhi;
@@ -471,7 +475,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
       // the chunk compares, accumulates a run of equal bins and flushes it on a change.
       constexpr int CH = (H + T - 1) / T;
       constexpr int NCH = (H + CH - 1) / CH;
-      static_assert(TX * NCH <= ColCfg<N>::THREADS, "one binning task per thread");
+      static_assert(TX * NCH <= ColCfg<N, MODE>::THREADS, "one binning task per thread");
       const int nb = a.nbins;
       const int tc = threadIdx.x % TX, ch = threadIdx.x / TX;
       const int gcol = col0 + tc;
@@ -497,7 +501,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
       }
       // natural order in shared memory
 #pragma unroll
-      for (int q = 0; q < E; ++q) line[p2pad(j + q * T)] = v[q];
+      for (int q = 0; q < E; ++q) line[p2pad<E>(j + q * T)] = v[q];
       __syncthreads();
       if (has) {
         const float2* ln = buf + tc * PITCH;
@@ -526,7 +530,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
             }
             if (b >= 0 && b < nb) {
               const float sc = a.vs ? csc * __ldg(a.vs + mm) : csc;
-              const float2 f1 = ln[p2pad(mm)];
+              const float2 f1 = ln[p2pad<E>(mm)];
               const float i1 = (f1.x * f1.x + f1.y * f1.y) * sc;
               if (fresh) {
                 K = ur_bin_shift(Kb, a.gK, b, i1);
@@ -536,7 +540,7 @@ __global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::MINB) k_p2_cols
               sI += d1;
               sI2 = fmaf(d1, d1, sI2);
               if (mm != 0 && mm != M) {
-                const float2 f2 = ln[p2pad(N - mm)];
+                const float2 f2 = ln[p2pad<E>(N - mm)];
                 const float d2 = (f2.x * f2.x + f2.y * f2.y) * sc - K;
                 sI += d2;
                 sI2 = fmaf(d2, d2, sI2);
@@ -733,37 +737,31 @@ bool ur_fast_supported(int n) {
   return n == 64 || n == 128 || n == 256 || n == 512 || n == 1024 || n == 2048 || n == 4096;
 }
 
-template <int N>
-static size_t cols_smem(int nbins, int mode) {
-  constexpr int TX = ColCfg<N>::TX, PITCH = P2<N>::PITCH + 2;
-  return ur_align_up((size_t)TX * PITCH * sizeof(float2), 16) + ur_align_up((size_t)(nbins + 1) * 4, 16) +
-         ur_align_up((size_t)nbins * 8, 16) + (mode == P2_Z_ADJ ? (size_t)UR_COARSE_ENTRIES * 2 : 0) +
-         (mode == P2_Z_BIN ? (size_t)nbins * 4 : 0);
+template <int N, int MODE>
+static ur_status launch_cols(const ColArgs& args, cudaStream_t s) {
+  using Cfg = ColCfg<N, MODE>;
+  ColArgs a = args;
+  if (Cfg::E == 32) a.stw = a.stw32;
+  const size_t nb = (size_t)a.nbins;
+  const size_t smem = ur_align_up((size_t)Cfg::TX * (P2<N, Cfg::E>::PITCH + 2) * sizeof(float2), 16) +
+                      ur_align_up((nb + 1) * 4, 16) + ur_align_up(nb * 8, 16) +
+                      (MODE == P2_Z_ADJ ? (size_t)UR_COARSE_ENTRIES * 2 : 0) + (MODE == P2_Z_BIN ? nb * 4 : 0);
+  const int grid = (int)((a.ncols + Cfg::TX - 1) / Cfg::TX);
+  if (grid <= 0) return UR_OK;
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_p2_cols<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_p2_cols<N, MODE><<<grid, Cfg::THREADS, smem, s>>>(a);
+  UR_LAUNCH_CHECK("k_p2_cols");
+  return UR_OK;
 }
 
 template <int N>
 static ur_status launch_cols_n(int mode, const ColArgs& a, cudaStream_t s) {
-  constexpr int TX = ColCfg<N>::TX;
-  const size_t smem = cols_smem<N>(a.nbins, mode);
-  const int grid = (int)((a.ncols + TX - 1) / TX);
-  if (grid <= 0) return UR_OK;
-#define UR_P2_LAUNCH(MD)                                                                                   \
-  do {                                                                                                     \
-    UR_CUDA_CHECK(cudaFuncSetAttribute(k_p2_cols<N, MD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-    k_p2_cols<N, MD><<<grid, ColCfg<N>::THREADS, smem, s>>>(a);                                                           \
-  } while (0)
   switch (mode) {
-    case P2_Y_FWD: UR_P2_LAUNCH(P2_Y_FWD); break;
-    case P2_Y_INV:
-      if (a.row_skip) UR_P2_LAUNCH(P2_Y_INV_ROWS);
-      else UR_P2_LAUNCH(P2_Y_INV);
-      break;
-    case P2_Z_BIN: UR_P2_LAUNCH(P2_Z_BIN); break;
-    default: UR_P2_LAUNCH(P2_Z_ADJ); break;
+    case P2_Y_FWD: return launch_cols<N, P2_Y_FWD>(a, s);
+    case P2_Y_INV: return a.row_skip ? launch_cols<N, P2_Y_INV_ROWS>(a, s) : launch_cols<N, P2_Y_INV>(a, s);
+    case P2_Z_BIN: return launch_cols<N, P2_Z_BIN>(a, s);
+    default: return launch_cols<N, P2_Z_ADJ>(a, s);
   }
-#undef UR_P2_LAUNCH
-  UR_LAUNCH_CHECK("k_p2_cols");
-  return UR_OK;
 }
 
 ur_status ur_fast_cols(int n, int mode, const ColArgs& a, cudaStream_t s) {

@@ -995,6 +995,7 @@ ColArgs ur_col_args(const ur_plan* p) {
   a.nst = p->sched_n.nst;
   a.tw = p->tw;
   a.stw = p->stw;
+  a.stw32 = p->stw + p->stw_32_off;
   a.thr = p->thr;
   a.lut = p->binlut;
   a.k2_zero = 0x7fffffff;

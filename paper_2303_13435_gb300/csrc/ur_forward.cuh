@@ -28,6 +28,7 @@ struct ColArgs {
   int nst;
   const float2* tw;
   const float2* stw;   // stage twiddles of the N-point transform (power-of-two kernels)
+  const float2* stw32; // ... with 32 values per thread
   // binning
   const int32_t* thr;
   const int16_t* lut;  // k^2 -> bin (-1 outside)

@@ -203,14 +203,14 @@ extern "C" int64_t ur_selftest_fastdiv(void) {
 }
 
 // Stage twiddles of the compile-time power-of-two transforms of length L = 2^lg
-// with E = 8 or 16 values per thread: radix-E Stockham stages (the last one of a
+// with E = 8, 16 or 32 values per thread: radix-E Stockham stages (the last one of a
 // smaller radix when lg is not a multiple of log2 E).  Stage S >= 1 has NS = E^S
 // butterfly classes k and radix R; its rows hold exp(-2 pi i r k / (NS R)) for
 // r < R at row k (E slots, unused ones 0), so a butterfly reads its R - 1
 // twiddles with at most E/2 16-byte loads.  Row blocks follow each other by
 // stage.  Returns the number of float2 written (out may be NULL to count).
 static size_t stage_twiddles(int lg, int E, float2* out) {
-  const int le = E == 16 ? 4 : 3;
+  const int le = E == 32 ? 5 : E == 16 ? 4 : 3;
   const int nfull = lg / le, rem = lg % le, nst = nfull + (rem ? 1 : 0);
   size_t off = 0;
   long long ns = 1;
@@ -425,21 +425,25 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
   if (ur_fast_supported(n)) {
     int lg = 0;
     while ((1 << lg) < n) ++lg;
-    // columns (N points): the pair table, or stages of UR_FAST_COL_E values per thread; rows (N/2
-    // points) 8, stored rows UR_FAST_STORED_ROW_E(n)
+    // tables, one after the other: columns (N points; pairs, or 16 values per thread), rows (N/2 points)
+    // with 8, stored rows where they take more, columns with 32
     const bool pair = ur_pair_supported(n);
-    const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : stage_twiddles(lg, UR_FAST_COL_E, nullptr);
-    const int erow = UR_FAST_STORED_ROW_E(n);
+    const int erow = UR_FAST_STORED_ROW_E(n), e32 = UR_FAST_COL_E(n, P2_Y_FWD);
+    const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : stage_twiddles(lg, 16, nullptr);
     const size_t cm = stage_twiddles(lg - 1, 8, nullptr), cs = erow == 8 ? 0 : stage_twiddles(lg - 1, erow, nullptr);
-    float2* st_h = (float2*)malloc(sizeof(float2) * (cn + cm + cs + 1));
+    const size_t c32 = e32 == 32 ? stage_twiddles(lg, 32, nullptr) : 0;
+    const size_t ct = cn + cm + cs + c32;
+    float2* st_h = (float2*)malloc(sizeof(float2) * (ct + 1));
     if (pair) ur_pair_twiddles(n, (float4*)st_h);
-    else stage_twiddles(lg, UR_FAST_COL_E, st_h);
+    else stage_twiddles(lg, 16, st_h);
     stage_twiddles(lg - 1, 8, st_h + cn);
     p->stw_m_off = (int)cn;
     p->stw_s_off = cs ? (int)(cn + cm) : p->stw_m_off;
     if (cs) stage_twiddles(lg - 1, erow, st_h + cn + cm);
-    const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (cn + cm + cs + 1));
-    const cudaError_t eb = ea == cudaSuccess ? cudaMemcpy(p->stw, st_h, sizeof(float2) * (cn + cm + cs + 1),
+    p->stw_32_off = (int)(cn + cm + cs);
+    if (c32) stage_twiddles(lg, 32, st_h + cn + cm + cs);
+    const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (ct + 1));
+    const cudaError_t eb = ea == cudaSuccess ? cudaMemcpy(p->stw, st_h, sizeof(float2) * (ct + 1),
                                                           cudaMemcpyHostToDevice) : ea;
     free(st_h);
     if (eb != cudaSuccess) {
