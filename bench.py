@@ -58,11 +58,11 @@ def peaks():
 # library kernel behind each timing label of the step (for the ncu profile lookup)
 KERNEL_OF = {
     "rows_r2c": "k_p2_rows<512, 1, float>",
-    "cols_y": "k_p2_cols<512, 0>",
-    "cols_z_bin": "k_p2_cols<512, 2>",
-    "adj_cols_z": "k_p2_cols<512, 3>",
-    "adj_cols_y": "k_p2_cols<512, 1>",
-    "adj_rows_grad": "k_p2_rows_grad<512>",
+    "cols_y": "k_pair_cols<512, 0>",
+    "cols_z_bin": "k_pair_cols<512, 2>",
+    "adj_cols_z": "k_pair_cols<512, 3>",
+    "adj_cols_y": "k_pair_cols<512, 1>",
+    "adj_rows_grad": "k_p2_rows_grad<512, 0>",
 }
 
 

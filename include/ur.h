@@ -114,8 +114,9 @@ void ur_fault_reset(void);
 enum { UR_WS_FORWARD = 1, UR_WS_BACKWARD = 2, UR_WS_HOST_SLABS = 4, UR_WS_ADJ_SLABS = 8 };
 /* Workspace bytes for the operations in `what` (bitwise OR of UR_WS_*).
  * The forward workspace holds the plane-transform intermediate
- * (nz * N * (N/2+1) complex64) and the per-block bin partials; the backward
- * adds the inverse intermediate (N * N * (N/2+1) complex64).  UR_WS_HOST_SLABS
+ * (nz * N * (N/2+1) complex64; power-of-two edges up to 512 pad its rows to 32
+ * bytes); the backward adds the inverse intermediate (N * N rows of the same
+ * length).  UR_WS_HOST_SLABS
  * adds two staging slabs for ED read from pinned host memory.  UR_WS_ADJ_SLABS
  * (ur_backward_slabs) adds, after the forward part and the host staging slabs
  * (counted whether or not UR_WS_HOST_SLABS is given), one slab of the inverse
@@ -242,8 +243,8 @@ ur_status ur_fft_intensity(const ur_plan* plan, const void* ed, int32_t ed_on_ho
  * [z0, z0+nz) is never stored.  cell, ucell, origin, shape and weights are
  * as for ur_build_density; the transform sees exactly the values
  * ur_build_density would write (FP32).  The plan's ed_dtype is ignored.
- * Cell values must be finite: a row whose mask is zero everywhere (a sphere
- * row outside the particle, or any row whose generated values are all zero)
+ * Cell values must be finite: a row whose mask is zero everywhere (a row
+ * outside the particle, or any row whose generated values are all zero)
  * is taken as zero without evaluating u * 0. */
 ur_status ur_fft_intensity_tiled(const ur_plan* plan, const float* cell, int32_t ucell, const int32_t* origin,
                                  const ur_shape* shape, const float* weights, double* bins, void* F_out, void* ws,
@@ -394,6 +395,8 @@ ur_status ur_ensemble_backward(int32_t count, const double* const* item_bins, co
  *   dl_dcell  device float32[U][U][U] (overwritten)
  *   dl_dmask  device float32[N][N][N] (overwritten), or NULL
  *   ws        the forward's workspace, sized with UR_WS_FORWARD | UR_WS_BACKWARD.
+ * With dl_dmask NULL only the planes and rows that the mask of a sphere, cube
+ * or octahedron can reach are transformed (dL/du needs no others).
  * dL/drho(x) = (2/N^3) Re sum_k G_k F_k exp(+2 pi i k.x/N), G_k = dl_dmean_j / count_j
  * on the voxels of bin j; dL/dm = dL/drho * u(x mod U); dL/du(c) = sum over the
  * tiles of dL/drho * m.

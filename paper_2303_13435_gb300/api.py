@@ -119,6 +119,7 @@ EXTRA = {
     "ur_selftest_fastdiv": (C.c_int64, []),
     "ur_selftest_dft": (C.c_double, []),
     "ur_selftest_wait_timeout": (_i32, [_vp]),
+    "ur_selftest_row_bound": (C.c_float, [C.POINTER(ShapeDesc)]),
 }
 
 _lib = None

@@ -194,6 +194,9 @@ extern "C" ur_status ur_build_density(int32_t n, const float* cell, int32_t ucel
                        stream);
 }
 
+// Test hook: the squared radius beyond which the rows of a shape are taken as outside (row_outside)
+extern "C" float ur_selftest_row_bound(const ur_shape* shape) { return ur_shape_args(shape).rb2; }
+
 extern "C" ur_status ur_build_density_lattice(int32_t n, const float* cell, int32_t ucell, const ur_lattice* lattice,
                                               const ur_shape* shape, const float* weights, int32_t z_begin,
                                               int32_t z_count, int32_t out_dtype, void* ed_out, int32_t* nz_range,
@@ -235,8 +238,8 @@ __device__ __forceinline__ unsigned short half_bits_from_fixed24(long long S) {
 }
 
 // FP16 block sums for f = 2, 4, 8, 16 and rows of whole 16-byte groups.  One block per output row
-// (Z, Y) of the particle, then blocks that zero the other rows; a thread sums the f^2 source rows of 8 neighbouring x.  Bound by the reads of the
-// source, so the exact integer sum must be cheap: with C = 1.5 2^17 every t = v + C lies in
+// (Z, Y) of the particle, then blocks that zero the other rows; a thread sums the f^2 source rows of 8
+// neighbouring x.  Bound by the reads of the source, so the exact integer sum must be cheap: with C = 1.5 2^17 every t = v + C lies in
 // [2^17, 2^18), where floats are multiples of 2^-6, so the bits of t count v rounded to 2^-6
 // (summed as int32) and v - (t - C), a multiple of 2^-24 of at most 2^-7, is summed exactly in
 // float32 over up to 128 terms before it is added to an integer.  A source row with an infinity or
