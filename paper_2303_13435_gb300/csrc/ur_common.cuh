@@ -674,8 +674,17 @@ __device__ __forceinline__ int bin_rank(const int16_t* crs, int shift, const int
 // (1 << 32) | float bits).  A block keeps the shifts it has seen in shared memory (NaN =
 // not yet fetched).  With K_j a value of the bin, the sums do not cancel when the
 // spread is small, so mean = K + S_d/n and M2 = Q_d - S_d^2/n stay accurate (Chan et
-// al.'s shifted-data form of the variance).
+// al.'s shifted-data form of the variance).  A K far above the bin's other values would cost
+// them their last bits, and the columns of ky = 0 are where such values lie (the kz axis of a
+// density cut by the box, or of few planes, reaches every bin), so the binned passes start with
+// the columns after them and take them last (ur_late_first_row).
 // ---------------------------------------------------------------------------
+// Block that block b of nblocks works on when the first `row` blocks come last
+__device__ __forceinline__ int ur_late_first_row(int b, int nblocks, int row) {
+  const int i = b + row;
+  return row >= nblocks ? b : i >= nblocks ? i - nblocks : i;
+}
+
 __device__ __forceinline__ float ur_bin_shift(float* Kb, unsigned long long* gK, int b, float v) {
   float k = Kb[b];
   if (k != k) {

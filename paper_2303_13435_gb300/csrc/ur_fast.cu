@@ -344,7 +344,8 @@ __global__ void __launch_bounds__((ColCfg<N, MODE>::THREADS), (ColCfg<N, MODE>::
                                             ur_align_up_dev((size_t)a.nbins * 8, 16));  // 16-byte aligned
   float* Kb = reinterpret_cast<float*>(crs);  // forward binning: the block's cache of the bin shifts
   const int c = threadIdx.x % TX, j = threadIdx.x / TX;
-  const int col0 = blockIdx.x * TX;
+  const int blk = MODE == P2_Z_BIN ? ur_late_first_row(blockIdx.x, gridDim.x, (H + TX - 1) / TX) : blockIdx.x;
+  const int col0 = blk * TX;
   const int col = col0 + c;
   const bool valid = col < a.ncols;
   const bool binning = (MODE == P2_Z_BIN || MODE == P2_Z_ADJ) && a.nbins > 0;

@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
   int16_t* crs = reinterpret_cast<int16_t*>(reinterpret_cast<unsigned char*>(hs) + ur_align_up_dev((size_t)nb * 8, 16));
   float* Kb = reinterpret_cast<float*>(crs);  // forward binning: the block's cache of the bin shifts
   const int c = threadIdx.x % TXP, j = threadIdx.x / TXP;
-  const int cp = blockIdx.x * TXP + c;
+  const int blk = MODE == P2_Z_BIN ? ur_late_first_row(blockIdx.x, gridDim.x, (CW + TXP - 1) / TXP) : blockIdx.x;
+  const int cp = blk * TXP + c;
   // row of the flattened index: |ky| in the z passes, plane pair in the y passes
   const int row = cp / CW, kx = cp - row * CW;
   const int ia = ZP ? row : 2 * row;
