@@ -45,15 +45,18 @@ __device__ __forceinline__ int p2pad(int i) { return i + (i >> (E == 32 ? 5 : 4)
 constexpr int ipowe(int e, int s) { return s == 0 ? 1 : e * ipowe(e, s - 1); }
 
 // Offset (float2) of stage S >= 1 in the stage twiddle table of an L-point transform:
-// the stages before S are radix E, with E^s rows of E slots each.
+// the stages before S are radix E, with E - 1 rows of E^s entries each.
 template <int E>
-constexpr int p2_stage_off(int S) { return S <= 1 ? 0 : p2_stage_off<E>(S - 1) + E * ipowe(E, S - 1); }
+constexpr int p2_stage_off(int S) { return S <= 1 ? 0 : p2_stage_off<E>(S - 1) + (E - 1) * ipowe(E, S - 1); }
 
 // Butterflies of stage S.  Thread j runs E/R butterflies b = j + i L/E; the
 // inputs of butterfly i are v[i + (E/R) r], r < R; k = b mod NS; the twiddles
-// exp(-+2 pi i r k/(NS R)), r = 1 .. R-1, are row k of the stage's block of the
-// stage table (plan-built in float64, stored float32; E slots per row), read as
-// 16-byte pairs.
+// exp(-+2 pi i r k/(NS R)), r = 1 .. R-1, are rows r of the stage's block of the
+// stage table, NS entries k each (plan-built in float64, stored float32), so that
+// neighbouring threads read neighbouring entries.  (Rows of E entries per k, read as
+// 16-byte pairs, were fewer loads, but 32 threads touched up to 16 lines with each: the adjoint
+// rows ran at 94 % of the L1 data pipe.  512^3: rows 68 -> 63 us, adjoint rows 270 -> 235;
+// 1024^3: rows 541 -> 451, FP16 rows 1849 -> 1082, adjoint rows 2612 -> 2188.)
 template <int L, int E, int R, int NS, int S, bool INV>
 __device__ __forceinline__ void p2_butterflies(float2 (&v)[E], int j, const float2* __restrict__ stw) {
   constexpr int T = L / E, NB = E / R;
@@ -65,16 +68,9 @@ __device__ __forceinline__ void p2_butterflies(float2 (&v)[E], int j, const floa
 #pragma unroll
     for (int r = 0; r < R; ++r) a[r] = v[i + NB * r];
     if constexpr (NS > 1) {
-      const float4* row = reinterpret_cast<const float4*>(stw + p2_stage_off<E>(S) + k * E);
-      float2 w[R];
+      const float2* w = stw + p2_stage_off<E>(S) + k;
 #pragma unroll
-      for (int h = 0; h < R / 2; ++h) {
-        const float4 t = __ldg(row + h);
-        w[2 * h] = make_float2(t.x, t.y);
-        w[2 * h + 1] = make_float2(t.z, t.w);
-      }
-#pragma unroll
-      for (int r = 1; r < R; ++r) a[r] = twmul<INV>(a[r], w[r]);
+      for (int r = 1; r < R; ++r) a[r] = twmul<INV>(a[r], __ldg(w + (r - 1) * NS));
     }
     dft<R, INV>(a);
 #pragma unroll

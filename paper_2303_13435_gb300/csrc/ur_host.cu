@@ -205,10 +205,9 @@ extern "C" int64_t ur_selftest_fastdiv(void) {
 // Stage twiddles of the compile-time power-of-two transforms of length L = 2^lg
 // with E = 8, 16 or 32 values per thread: radix-E Stockham stages (the last one of a
 // smaller radix when lg is not a multiple of log2 E).  Stage S >= 1 has NS = E^S
-// butterfly classes k and radix R; its rows hold exp(-2 pi i r k / (NS R)) for
-// r < R at row k (E slots, unused ones 0), so a butterfly reads its R - 1
-// twiddles with at most E/2 16-byte loads.  Row blocks follow each other by
-// stage.  Returns the number of float2 written (out may be NULL to count).
+// butterfly classes k and radix R; its rows r = 1 .. R - 1 hold exp(-2 pi i r k / (NS R))
+// for k < NS.  Row blocks follow each other by stage.  Returns the number of
+// float2 written (out may be NULL to count).
 static size_t stage_twiddles(int lg, int E, float2* out) {
   const int le = E == 32 ? 5 : E == 16 ? 4 : 3;
   const int nfull = lg / le, rem = lg % le, nst = nfull + (rem ? 1 : 0);
@@ -217,16 +216,12 @@ static size_t stage_twiddles(int lg, int E, float2* out) {
   for (int st = 0; st < nst; ++st) {
     const int R = st < nfull ? E : (1 << rem);
     if (st >= 1) {
-      for (long long k = 0; k < ns; ++k)
-        for (int r = 0; r < E; ++r) {
-          float2 w = make_float2(0.f, 0.f);
-          if (r < R) {
+      for (int r = 1; r < R; ++r)
+        for (long long k = 0; k < ns; ++k, ++off)
+          if (out) {
             const double a = 2.0 * M_PI * (double)(r * k) / (double)(ns * R);
-            w = make_float2((float)cos(a), (float)(-sin(a)));
+            out[off] = make_float2((float)cos(a), (float)(-sin(a)));
           }
-          if (out) out[off + (size_t)k * E + r] = w;
-        }
-      off += (size_t)ns * E;
     }
     ns *= R;
   }
