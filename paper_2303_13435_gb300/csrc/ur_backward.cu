@@ -535,7 +535,7 @@ ur_status ur_batch_launch_grad(const BatchGradItem* items, const long long* star
                                size_t smem, cudaStream_t s) {
   if (nblocks <= 0) return UR_OK;
   UR_REQUIRE(nblocks < (1ll << 31), "batched adjoint rows: too many blocks");
-  if (smem > 48 * 1024)
+  if (smem > UR_DYN_SMEM_FREE)
     UR_CUDA_CHECK(cudaFuncSetAttribute(k_batch_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_batch_grad<<<(unsigned)nblocks, 256, smem, s>>>(items, start, count);
   UR_LAUNCH_CHECK("k_batch_grad");

@@ -49,6 +49,10 @@ ur_status ur_fault_point(const char* site);  // host-side fault injection (UR_FA
     if (ur_s_ != UR_OK) return ur_s_;     \
   } while (0)
 
+// Dynamic shared memory that a kernel may be launched with before its limit is raised: the default
+// of 48 KB holds the kernel's static variables too (at most 1 KB in the kernels that use this).
+#define UR_DYN_SMEM_FREE (47 * 1024)
+
 // ---------------------------------------------------------------------------
 // Division by a run-time constant: q = (umulhi(x, m) + x) >> s with
 // s = ceil(log2 d), m = floor(2^32 (2^s - d) / d) + 1 (Granlund & Montgomery,

@@ -456,7 +456,7 @@ static ur_status launch_pair(const ColArgs& args, cudaStream_t s) {
   const size_t nb = (size_t)a.nbins;
   const size_t smem = (size_t)Cfg::TXP * Cfg::PITCH * 16 + ur_align_up((nb + 1) * 4, 16) + ur_align_up(nb * 8, 16) +
                       (MODE == P2_Z_ADJ ? (size_t)UR_COARSE_ENTRIES * 2 : 0) + (MODE == P2_Z_BIN ? nb * 4 : 0);
-  if (smem > 48 * 1024)
+  if (smem > UR_DYN_SMEM_FREE)
     UR_CUDA_CHECK(cudaFuncSetAttribute(k_pair_cols<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_pair_cols<N, MODE><<<(unsigned)blocks, Cfg::THREADS, smem, s>>>(a);
   UR_LAUNCH_CHECK("k_pair_cols");
