@@ -120,6 +120,7 @@ EXTRA = {
     "ur_selftest_dft": (C.c_double, []),
     "ur_selftest_wait_timeout": (_i32, [_vp]),
     "ur_selftest_row_bound": (C.c_float, [C.POINTER(ShapeDesc)]),
+    "ur_selftest_row_ranges": (None, [C.POINTER(ShapeDesc), _i32, C.POINTER(_i32)]),
 }
 
 _lib = None

@@ -197,6 +197,16 @@ extern "C" ur_status ur_build_density(int32_t n, const float* cell, int32_t ucel
 // Test hook: the squared radius beyond which the rows of a shape are taken as outside (row_outside)
 extern "C" float ur_selftest_row_bound(const ur_shape* shape) { return ur_shape_args(shape).rb2; }
 
+// Test hook: the rows of planes 0 .. n - 1 that the column passes take as the particle's, (first, count) pairs
+extern "C" void ur_selftest_row_ranges(const ur_shape* shape, int32_t n, int32_t* out) {
+  const ShapeArgs sh = ur_shape_args(shape);
+  for (int z = 0; z < n; ++z) {
+    const int2 r = row_range(sh, z, n);
+    out[2 * z] = r.x;
+    out[2 * z + 1] = r.y;
+  }
+}
+
 extern "C" ur_status ur_build_density_lattice(int32_t n, const float* cell, int32_t ucell, const ur_lattice* lattice,
                                               const ur_shape* shape, const float* weights, int32_t z_begin,
                                               int32_t z_count, int32_t out_dtype, void* ed_out, int32_t* nz_range,

@@ -122,12 +122,41 @@ struct RowMask {
 // to nearest is monotone and fl(dx*dx) >= 0, so fl(fl(fl(dx*dx) + dy2) + dz2) >= fl(dy2 + dz2) for
 // every x.  Cube and octahedron: rb2 is the square of a radius beyond their vertices
 // (ur_shape_args).
-__device__ __forceinline__ bool row_outside(float cy, float cz, float rb2, int y, int z) {
+// (Host-callable, for row_range and its test; the volatile results keep the host compiler from
+// contracting the product and the sum.)
+UR_HD __forceinline__ bool row_outside(float cy, float cz, float rb2, int y, int z) {
+#ifdef __CUDA_ARCH__
   const float dy = __fsub_rn((float)y, cy), dz = __fsub_rn((float)z, cz);
   return __fadd_rn(__fmul_rn(dy, dy), __fmul_rn(dz, dz)) > rb2;
+#else
+  const volatile float dy = (float)y - cy, dz = (float)z - cz;
+  const volatile float dy2 = dy * dy, dz2 = dz * dz;
+  const volatile float d2 = dy2 + dz2;
+  return d2 > rb2;
+#endif
 }
-__device__ __forceinline__ bool row_outside(const ShapeArgs& sh, int y, int z) {
+UR_HD __forceinline__ bool row_outside(const ShapeArgs& sh, int y, int z) {
   return row_outside(sh.cy, sh.cz, sh.rb2, y, z);
+}
+
+// Rows y of plane z that the particle can reach, (first, count): those that row_outside does not take
+// as outside.  They are neighbours, since row_outside is monotone on either side of the centre.  The
+// square root is only where the search starts: the walks inwards drop what is outside, the walks
+// outwards find rows of spheres so large (from about 2^14 voxels radius) that the float32 steps of
+// rb2 are wider than the margin of the start.  For other particles each walk ends at its first or
+// second step.
+UR_HD __forceinline__ int2 row_range(const ShapeArgs& sh, int z, int N) {
+  const float dz = (float)z - sh.cz;
+  const float r = sqrtf(fmaxf(sh.rb2 - dz * dz, 0.f));
+  int a = (int)floorf(fminf(fmaxf(sh.cy - r, -1.f), (float)N)) - 1;
+  int b = (int)ceilf(fminf(fmaxf(sh.cy + r, -2.f), (float)N)) + 1;
+  a = a > 0 ? a : 0;
+  b = b < N - 1 ? b : N - 1;
+  while (a > 0 && !row_outside(sh, a - 1, z)) --a;
+  while (b < N - 1 && !row_outside(sh, b + 1, z)) ++b;
+  while (a <= b && row_outside(sh, a, z)) ++a;
+  while (b >= a && row_outside(sh, b, z)) --b;
+  return make_int2(a, b >= a ? b - a + 1 : 0);
 }
 
 // Rotated lattice (Sec. 2.3: the cell sampled on rotated planes with periodic wrap).

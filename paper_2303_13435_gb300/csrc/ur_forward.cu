@@ -265,18 +265,6 @@ struct ColSt {
   }
 };
 
-// Rows y of plane z that the particle can reach, (first, count): row_outside is monotone on either
-// side of the centre, so the square root's neighbourhood decides it exactly.
-__device__ __forceinline__ int2 row_range(const ShapeArgs& sh, int z, int N) {
-  const float dz = __fsub_rn((float)z, sh.cz);
-  const float r = sqrtf(fmaxf(sh.rb2 - dz * dz, 0.f));
-  int a = max(0, (int)floorf(fminf(fmaxf(sh.cy - r, -1.f), 1e6f)) - 1);
-  int b = min(N - 1, (int)ceilf(fminf(fmaxf(sh.cy + r, -2.f), 1e6f)) + 1);
-  while (a <= b && row_outside(sh, a, z)) ++a;
-  while (b >= a && row_outside(sh, b, z)) --b;
-  return make_int2(a, max(b - a + 1, 0));
-}
-
 // Elements i of a column of kx that lie at or beyond k2_zero, (first, count): |ky| > km, the largest
 // with kx^2 + km^2 < k2_zero, is i in (km, N - km)
 __device__ __forceinline__ int2 beyond_range(int kx, int k2_zero, int N) {
