@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
       static_assert(CH * T == M, "whole chunks");
       const bool has = valid;
       const int m0 = j * CH;
-      const float w = (kx == 0 || kx == M) ? 1.f : 2.f, wb = hasb ? w : 0.f;
+      const float w = (kx == 0 || kx == M) ? 1.f : 2.f;
       float csc = a.iscale;  // I scale of the pair (times its voxel-sinc factor)
       int b = -1;
       if (has) {
@@ -345,8 +345,9 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
         bool fresh = true;
         auto flush = [&]() {
           const float2 t = f2_get(sI), t2 = f2_get(sI2);
-          atomicAdd(hs + b, w * t.x + wb * t.y);
-          atomicAdd(hs2 + b, w * t2.x + wb * t2.y);
+          // without a partner lane B holds (0 - K)^2, which may have overflowed: left out, not weighed with 0
+          atomicAdd(hs + b, w * (hasb ? t.x + t.y : t.x));
+          atomicAdd(hs2 + b, w * (hasb ? t2.x + t2.y : t2.x));
           sI = sI2 = 0ull;
           fresh = true;
         };
