@@ -178,9 +178,11 @@ def _torch_dtype(code: int):
 
 
 def shape_desc(shape) -> ShapeDesc:
-    c = np.asarray(shape.center, dtype=np.float32).tolist()
+    # the first three coordinates: a shorter centre is an IndexError
+    c = np.asarray(shape.center, dtype=np.float32)
+    c = (C.c_float * 3)(float(c[0]), float(c[1]), float(c[2]))
     r = np.asarray(shape.rot, dtype=np.float32).reshape(9).tolist()
-    return ShapeDesc(int(shape.kind), (C.c_float * 3)(*c), float(np.float32(shape.size)), (C.c_float * 9)(*r))
+    return ShapeDesc(int(shape.kind), c, float(np.float32(shape.size)), (C.c_float * 9)(*r))
 
 
 class Plan:
