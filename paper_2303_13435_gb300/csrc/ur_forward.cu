@@ -1269,7 +1269,7 @@ ur_status ur_batch_launch_rows(const BatchRowsItem* items, const long long* star
   if (nblocks <= 0) return UR_OK;
   UR_REQUIRE(nblocks < (1ll << 31), "batched rows: too many blocks");
   batch_grid_check(nblocks);
-  if (smem > 48 * 1024)
+  if (smem > UR_DYN_SMEM_FREE)
     UR_CUDA_CHECK(cudaFuncSetAttribute(k_batch_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_batch_rows<<<(unsigned)nblocks, 256, smem, s>>>(items, start, count);
   UR_LAUNCH_CHECK("k_batch_rows");

@@ -44,3 +44,20 @@ b.dl_dmean[0].fill_(1.0)
 b.backward()
 assert torch.isfinite(b.dl_dcell[0]).all() and b.dl_dcell[0].abs().sum().item() > 0
 """)
+
+
+def test_batched_rows():
+    # 256 rows of 32: 48 KB of lines and row terms, and the stage table beside them
+    run("""
+import torch
+from paper_2303_13435_gb300 import api, inputs
+plan = api.Plan(32, 0.05, inputs.linear_edges(inputs.nyquist_q(0.05), 20))
+plan.set_tiles(256, 0)
+cell = torch.rand((6, 6, 6), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+shape = inputs.Shape(inputs.SHAPE_SPHERE, (16.0, 16.0, 16.0), 12.0)
+b = api.Batch([plan], cell, [shape])
+bins = b.forward()[0]
+one = api.fft_intensity_tiled(api.Plan(32, 0.05, plan.edges), cell, shape)
+ok = bins[api.BIN_COUNT] > 0
+assert torch.allclose(bins[api.BIN_MEAN][ok], one[api.BIN_MEAN][ok], rtol=1e-5)
+""")
