@@ -158,10 +158,18 @@ def _ptr(t) -> int | None:
     return t.data_ptr()
 
 
+def _raw_stream_of():
+    """Handle of a device's current stream: torch's internal accessor, which builds no torch.cuda.Stream
+    around it, or the public call in a version without it."""
+    return getattr(torch._C, "_cuda_getCurrentRawStream", lambda d: torch.cuda.current_stream(d).cuda_stream)
+
+
+_raw_stream = _raw_stream_of()
+
+
 def _stream(stream) -> int | None:
     if stream is None:
-        # the raw handle of the current stream, without building a torch.cuda.Stream around it
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
