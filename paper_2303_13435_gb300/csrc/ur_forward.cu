@@ -1196,10 +1196,19 @@ extern "C" ur_status ur_bin_q(const ur_plan* p, const float* I, double* bins, vo
   a.nb = nb;
   // long walks merge more elements per histogram update, short ones fill the GPU on small grids:
   // 16 steps per task (512^3: 64 steps 291 us, 32 199, 16 184, 8 186) while that leaves two tasks per
-  // resident thread, never fewer than 4
+  // resident thread, and 8 or 4 below; 2 and 1, in blocks of half the size, where walks of 4 give less
+  // than 512 threads per SM (below about 130^3), us with 40, 300, 771, 1000 bins (40 and 771: log):
+  //           4 steps, 256 threads     2 or 1 steps, 128 threads
+  //    48^3   23.4 17.1 29.0 21.4      14.4 10.9 12.2 12.6
+  //    84^3   27.0 17.3 26.5 20.1      18.5 12.7 15.0 16.3
+  //   126^3   31.3 21.0 26.6 21.2      23.1 16.9 18.3 20.6
+  //   160^3   37.7 25.2 27.9 25.1      34.5 23.6 25.9 27.8
   const long long ncol = (long long)p->H * p->H;
+  auto tasks = [&] { return ncol * ((p->H + a.chunk - 1) / a.chunk); };
   a.chunk = 16;
-  while (a.chunk > 4 && ncol * ((p->H + a.chunk - 1) / a.chunk) < (long long)p->num_sms * 2048) a.chunk /= 2;
+  while (a.chunk > 4 && tasks() < (long long)p->num_sms * 2048) a.chunk /= 2;
+  while (a.chunk > 1 && tasks() < (long long)p->num_sms * 512) a.chunk /= 2;
+  const int threads = a.chunk < 4 ? UR_BINQ_THREADS / 2 : UR_BINQ_THREADS;
   a.nchunk = (p->H + a.chunk - 1) / a.chunk;
   a.thr = p->thr;
   a.lut = p->binlut;
@@ -1211,11 +1220,11 @@ extern "C" ur_status ur_bin_q(const ur_plan* p, const float* I, double* bins, vo
   a.f1 = n3 / s2;
   a.f2 = (n3 / s2) * (n3 / s2);
   a.vs = p->vsinc;
-  const long long need = (ncol * a.nchunk + UR_BINQ_THREADS - 1) / UR_BINQ_THREADS;
+  const long long need = (tasks() + threads - 1) / threads;
   const int cap = p->num_sms * (smem > 40 * 1024 ? 1 : 4);
   const int grid = (int)(need < cap ? need : cap);
-  if (a.vs) k_bin_half<true><<<grid, UR_BINQ_THREADS, smem, s>>>(a);
-  else k_bin_half<false><<<grid, UR_BINQ_THREADS, smem, s>>>(a);
+  if (a.vs) k_bin_half<true><<<grid, threads, smem, s>>>(a);
+  else k_bin_half<false><<<grid, threads, smem, s>>>(a);
   UR_LAUNCH_CHECK("k_bin_half");
   k_finalize<<<(nb + 255) / 256, 256, 0, s>>>(bins, p->geo, nb, 1.0 / n3);
   UR_LAUNCH_CHECK("k_finalize");
