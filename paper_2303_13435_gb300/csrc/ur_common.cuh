@@ -141,6 +141,7 @@ __device__ __forceinline__ ur_f2 f2_mul(ur_f2 a, ur_f2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ ur_f2 f2_neg(ur_f2 a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ ur_f2 f2_fma(ur_f2 a, ur_f2 b, ur_f2 c) {
   ur_f2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));

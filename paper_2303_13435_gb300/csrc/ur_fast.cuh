@@ -62,6 +62,7 @@ bool ur_fast_supported(int n);
 ur_status ur_fast_rows(int n, const RowArgs& a, int gen, int ed_f16, cudaStream_t s);
 ur_status ur_fast_cols(int n, int mode, const ColArgs& a, cudaStream_t s);
 bool ur_pair_supported(int n);
+size_t ur_stage_twiddles(int lg, int E, float2* out);
 size_t ur_pair_twiddles(int n, float4* out);
 ur_status ur_pair_cols(int n, int mode, const ColArgs& a, cudaStream_t s);
 ur_status ur_fast_rows_grad(int n, const GradArgs& a, int nplanes, cudaStream_t s);

@@ -226,7 +226,7 @@ static double dft_gain_of(int R) { return R == 8 ? dft_gain<8>() : R == 16 ? dft
 // smaller radix when lg is not a multiple of log2 E).  Stage S >= 1 has NS = E^S
 // butterfly classes k and radix R; its rows r = 1 .. R - 1 hold exp(-2 pi i r k / (NS R))
 // for k < NS.  Row blocks follow each other by stage.  Returns the number of
-// float2 written (out may be NULL to count).
+// float2 written (out may be NULL to count; ur_pair_twiddles stores the same entries twice over).
 //
 // Each stage's entries are scaled by a few 1e-8 before they are rounded, so that the stage (and for
 // S = 1 stage 0 with it) has a mean gain of 1: without that the roundings of the constants add up to a
@@ -234,7 +234,7 @@ static double dft_gain_of(int R) { return R == 8 ? dft_gain<8>() : R == 16 ? dft
 // multiply, and the longer radices were less accurate by it.  Error of white noise against float64,
 // normwise: 512 values 1.00e-7 -> 0.98e-7 (8, 8, 8), 1.03 -> 1.00 (16, 16, 2); 1024 values 1.08 -> 1.06
 // (16, 16, 4), 1.11 -> 1.04 (32, 32).
-static size_t stage_twiddles(int lg, int E, float2* out) {
+size_t ur_stage_twiddles(int lg, int E, float2* out) {
   const int le = E == 32 ? 5 : E == 16 ? 4 : 3;
   const int nfull = lg / le, rem = lg % le, nst = nfull + (rem ? 1 : 0);
   size_t off = 0;
@@ -464,19 +464,19 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
     // with 8, stored rows where they take more, columns with 32
     const bool pair = ur_pair_supported(n);
     const int erow = UR_FAST_STORED_ROW_E(n), e32 = UR_FAST_COL_E(n, P2_Y_FWD);
-    const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : stage_twiddles(lg, 16, nullptr);
-    const size_t cm = stage_twiddles(lg - 1, 8, nullptr), cs = erow == 8 ? 0 : stage_twiddles(lg - 1, erow, nullptr);
-    const size_t c32 = e32 == 32 ? stage_twiddles(lg, 32, nullptr) : 0;
+    const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : ur_stage_twiddles(lg, 16, nullptr);
+    const size_t cm = ur_stage_twiddles(lg - 1, 8, nullptr), cs = erow == 8 ? 0 : ur_stage_twiddles(lg - 1, erow, nullptr);
+    const size_t c32 = e32 == 32 ? ur_stage_twiddles(lg, 32, nullptr) : 0;
     const size_t ct = cn + cm + cs + c32;
     float2* st_h = (float2*)malloc(sizeof(float2) * (ct + 1));
     if (pair) ur_pair_twiddles(n, (float4*)st_h);
-    else stage_twiddles(lg, 16, st_h);
-    stage_twiddles(lg - 1, 8, st_h + cn);
+    else ur_stage_twiddles(lg, 16, st_h);
+    ur_stage_twiddles(lg - 1, 8, st_h + cn);
     p->stw_m_off = (int)cn;
     p->stw_s_off = cs ? (int)(cn + cm) : p->stw_m_off;
-    if (cs) stage_twiddles(lg - 1, erow, st_h + cn + cm);
+    if (cs) ur_stage_twiddles(lg - 1, erow, st_h + cn + cm);
     p->stw_32_off = (int)(cn + cm + cs);
-    if (c32) stage_twiddles(lg, 32, st_h + cn + cm + cs);
+    if (c32) ur_stage_twiddles(lg, 32, st_h + cn + cm + cs);
     const cudaError_t ea = cudaMalloc(&p->stw, sizeof(float2) * (ct + 1));
     const cudaError_t eb = ea == cudaSuccess ? cudaMemcpy(p->stw, st_h, sizeof(float2) * (ct + 1),
                                                           cudaMemcpyHostToDevice) : ea;

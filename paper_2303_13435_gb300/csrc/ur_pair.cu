@@ -22,8 +22,7 @@
 // (y 932 -> 985, adjoint z 2538 -> 2684; z + bins of a full grid 2231 -> 2510 us: rows ky and -ky of a
 // plane lie in different 2 MB pages), so from 1024 on the columns are transformed one by one
 // (ur_fast.cu).
-#include <math.h>
-#include <string.h>
+#include <vector>
 
 #include "ur_fast.cuh"
 
@@ -41,12 +40,12 @@ template <bool INV>
 __device__ __forceinline__ C2 c2_sub_ni(C2 a, C2 b) {
   return c2_add_ni<!INV>(a, b);
 }
-// a * w, w = (wx, wx, wy, wy) the forward twiddle (inverse: its conjugate)
+// a * w, w = (wx, wx, wy, wy) the forward twiddle (inverse: its conjugate); both components end in a
+// fused multiply-add, so that one product of each is not rounded
 template <bool INV>
 __device__ __forceinline__ C2 c2_twmul(C2 a, ulonglong2 w) {
-  const ur_f2 p = f2_mul(a.x, w.x), q = f2_mul(a.y, w.x);
-  if constexpr (INV) return {f2_fma(a.y, w.y, p), f2_sub(q, f2_mul(a.x, w.y))};
-  else return {f2_sub(p, f2_mul(a.y, w.y)), f2_fma(a.x, w.y, q)};
+  const ur_f2 p = f2_mul(a.x, w.x), q = f2_mul(a.y, w.x), n = f2_neg(w.y);
+  return INV ? C2{f2_fma(a.y, w.y, p), f2_fma(a.x, n, q)} : C2{f2_fma(a.y, n, p), f2_fma(a.x, w.y, q)};
 }
 template <bool INV>
 __device__ __forceinline__ void c2_dft4(C2& a0, C2& a1, C2& a2, C2& a3) {
@@ -426,23 +425,16 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
 // ---------------------------------------------------------------------------
 bool ur_pair_supported(int n) { return n == 64 || n == 128 || n == 256 || n == 512; }
 
-// Twiddle table of the N-point column transform: for stage S >= 1 of radix R with NS = E^S classes,
-// rows r = 1 .. R - 1 of NS entries (wx, wx, wy, wy), w = exp(-2 pi i r k / (NS R)) from float64.
-// Returns the number of 16-byte words (out may be NULL to count).
+// Twiddle table of the N-point column transform: the entries w of ur_stage_twiddles for 8 values per
+// thread as (wx, wx, wy, wy).  Returns the number of 16-byte words (out may be NULL to count).
 size_t ur_pair_twiddles(int n, float4* out) {
-  const int log = pair_log(n), le = 3;
-  size_t off = 0;
-  for (int S = 1; S * le < log; ++S) {
-    const int R = pair_radix(log, le, S), NS = pair_pow(1 << le, S);
-    for (int r = 1; r < R; ++r)
-      for (int k = 0; k < NS; ++k, ++off) {
-        if (!out) continue;
-        const double t = 2.0 * M_PI * (double)(r * k) / (double)(NS * R);
-        const float wx = (float)cos(t), wy = (float)(-sin(t));
-        out[off] = make_float4(wx, wx, wy, wy);
-      }
+  const size_t cnt = ur_stage_twiddles(pair_log(n), 8, nullptr);
+  if (out) {
+    std::vector<float2> w(cnt);
+    ur_stage_twiddles(pair_log(n), 8, w.data());
+    for (size_t i = 0; i < cnt; ++i) out[i] = make_float4(w[i].x, w[i].x, w[i].y, w[i].y);
   }
-  return off;
+  return cnt;
 }
 
 template <int N, int MODE>
