@@ -693,9 +693,9 @@ ur_status ur_launch_geometry(ur_plan* p, cudaStream_t s) {
 // together.  A float64 instruction occupies its pipe for a whole warp however few lanes are
 // active, so float64 comes last: runs are three-float sums (72 bits) of the intensity scaled
 // by a power of two, finished runs are queued per warp, and 32 of them at a time are added to
-// the block's float64 histogram (compare-and-swap loops).  A value outside the range where its
-// square and the square's rounding error are both representable goes to the histogram in
-// float64 by itself.  512^3, 512 bins: 1918 us with one element per thread (64-bit division,
+// the block's float64 histogram (compare-and-swap loops).  Values outside the range where their
+// squares and the squares' rounding errors are both representable go to the histogram in float64,
+// summed over a step.  512^3, 512 bins: 1918 us with one element per thread (64-bit division,
 // binary search, two float64 histogram updates), 361 us with runs over (+-n, +-m) that each
 // lane adds to the histogram itself (float64 pipe 77 % busy), 184 us now (kernel 168 us, 1.7 TB/s, 62 % issue).
 // ---------------------------------------------------------------------------
@@ -810,20 +810,21 @@ __global__ void __launch_bounds__(UR_BINQ_THREADS, 4) k_bin_half(const __grid_co
     };
     for (int y = ylo; y < yhi; y += UR_BINQ_STEPS) {
       float v[UR_BINQ_STEPS][8];
+      auto value = [&](int n, int e, bool in) {
+        const bool two = n != 0 && n != M, swap = n != m;
+        const float* p = e < 4 ? (e & 2 ? pz1 : pz0) : (e & 2 ? py1 : py0);
+        const long long o = (long long)(e & 1 ? N - n : n) * H * (e < 4 ? 1 : N);
+        return in && (!(e & 1) || two) && (!(e & 2) || twom) && (!(e & 4) || swap) ? __ldg(p + o) : 0.f;
+      };
+      // x^2 of x = v s and its rounding error are both normal floats, or zero
+      auto in_range = [&](float v) {
+        const float x = fabsf(v * a.s);
+        return x <= 1e18f && (x >= 1e-15f || v == 0.f);
+      };
 #pragma unroll
-      for (int u = 0; u < UR_BINQ_STEPS; ++u) {
-        const int n = y + u;
-        const bool in = n >= y0 && n < y1, two = in && n != 0 && n != M, swap = n != m;
-        const long long o0 = (long long)n * H, o1 = (long long)(N - n) * H;
-        v[u][0] = in ? __ldg(pz0 + o0) : 0.f;
-        v[u][1] = two ? __ldg(pz0 + o1) : 0.f;
-        v[u][2] = in && twom ? __ldg(pz1 + o0) : 0.f;
-        v[u][3] = two && twom ? __ldg(pz1 + o1) : 0.f;
-        v[u][4] = in && swap ? __ldg(py0 + o0 * N) : 0.f;
-        v[u][5] = two && swap ? __ldg(py0 + o1 * N) : 0.f;
-        v[u][6] = in && swap && twom ? __ldg(py1 + o0 * N) : 0.f;
-        v[u][7] = two && swap && twom ? __ldg(py1 + o1 * N) : 0.f;
-      }
+      for (int u = 0; u < UR_BINQ_STEPS; ++u)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[u][e] = value(y + u, e, y + u >= y0 && y + u < y1);
 #pragma unroll
       for (int u = 0; u < UR_BINQ_STEPS; ++u) {
         const int n = y + u;
@@ -840,12 +841,12 @@ __global__ void __launch_bounds__(UR_BINQ_THREADS, 4) k_bin_half(const __grid_co
           // voxel-sinc factors in the order (x y) z
           const float vn = VS ? __ldg(a.vs + n) : 0.f;
           const float fa = VS ? vx * vn * vm : 1.f, fb = VS ? vx * vm * vn : 1.f;
+          bool all = true;
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const float f = e < 4 ? fa : fb;
             const float x = v[u][e] * a.s;
-            // |x| in [1e-15, 1e18], or zero: x^2 and its rounding error are both normal floats
-            if (fabsf(x) <= 1e18f && (fabsf(x) >= 1e-15f || v[u][e] == 0.f)) {
+            if (in_range(v[u][e])) {
               float p = x, r = 0.f;
               if (VS) {
                 p = __fmul_rn(x, f);
@@ -862,11 +863,22 @@ __global__ void __launch_bounds__(UR_BINQ_THREADS, 4) k_bin_half(const __grid_co
                 s2.e += fmaf(r, r, __fmaf_rn(2.f * p, r, -pr));
               }
             } else {
-              double d = (double)v[u][e] * a.sd;
-              if (VS) d *= (double)f;
-              atomicAdd(hs + b, (double)w * d);
-              atomicAdd(hs2 + b, (double)w * d * d);
+              all = false;
             }
+          }
+          if (!all) {  // the step's other values, read once more: one float64 sum
+            double d1 = 0.0, d2 = 0.0;
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+              const float t = value(n, e, true);
+              if (in_range(t)) continue;
+              double d = (double)t * a.sd;
+              if (VS) d *= (double)(e < 4 ? fa : fb);
+              d1 += d;
+              d2 += d * d;
+            }
+            atomicAdd(hs + b, (double)w * d1);
+            atomicAdd(hs2 + b, (double)w * d2);
           }
         }
         if (in) s += 2 * n + 1;

@@ -47,3 +47,24 @@ def time(plan, half):
 def test_a_smaller_grid_takes_less_time():
     # 48^3 has a sixteenth of the elements of 126^3; with serial walks of four steps it took longer
     assert time(*setup(48, 771)) < 0.9 * time(*setup(126, 771))
+
+
+def test_the_unit_does_not_matter():
+    """Values of 1e-30 took the histogram's float64 additions one by one, which was nine times as long; summed
+    over the eight values of a step it has to be less than three times as long."""
+    plan, half = setup(128, 40)
+    assert time(plan, half * 1e-30) < 3 * time(plan, half)
+
+
+@pytest.mark.parametrize("n", [8, 48, 140])
+@pytest.mark.parametrize("power", [-140, -120, -100, -60, 60, 90, 120])
+def test_scaled_sums(n, power):
+    """An intensity times a power of two: sums of runs held to 48 bits, so 1e-12, on either scale."""
+    plan, half = setup(n, 60)
+    half = (half * 2.0 ** min(power, 0)).float().double() * 2.0 ** -min(power, 0)  # exact where it is subnormal
+    half[0, 0, 0] *= 2.0 ** 6
+    want = api.bin_q(plan, half.float())
+    got = api.bin_q(plan, (half * 2.0 ** power).float())
+    assert torch.equal(got[api.BIN_COUNT], want[api.BIN_COUNT])
+    for f, p in ((api.BIN_SUM_I, power), (api.BIN_SUM_I2, 2 * power)):
+        assert torch.allclose(got[f] * 2.0 ** -p, want[f], rtol=1e-12, atol=0)
