@@ -50,8 +50,8 @@ ur_status ur_fault_point(const char* site);  // host-side fault injection (UR_FA
   } while (0)
 
 // Dynamic shared memory that a kernel may be launched with before its limit is raised: the default
-// of 48 KB holds the kernel's static variables too (at most 1 KB in the kernels that use this).
-#define UR_DYN_SMEM_FREE (47 * 1024)
+// of 48 KB holds the kernel's static variables too (at most 1136 bytes in the kernels that use this).
+#define UR_DYN_SMEM_FREE (46 * 1024)
 
 // ---------------------------------------------------------------------------
 // Division by a run-time constant: q = (umulhi(x, m) + x) >> s with

@@ -30,15 +30,16 @@ assert bins[1].sum().item() > 0
 """)
 
 
-def test_batched_adjoint_rows():
-    # 195 rows of 42: 48.0 KB of lines, row terms and counts
-    run("""
+# 195 rows of 42: 48.0 KB of lines, row terms and counts; 197 of 40: 47.0 KB, and 1136 bytes of static variables
+@pytest.mark.parametrize("n,rows", [(42, 195), (40, 197)])
+def test_batched_adjoint_rows(n, rows):
+    run(f"""
 import torch
 from paper_2303_13435_gb300 import api, inputs
-plan = api.Plan(42, 0.05, inputs.linear_edges(inputs.nyquist_q(0.05), 20))
-plan.set_tiles(195, 0)
+plan = api.Plan({n}, 0.05, inputs.linear_edges(inputs.nyquist_q(0.05), 20))
+plan.set_tiles({rows}, 0)
 cell = torch.rand((6, 6, 6), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
-b = api.Batch([plan], cell, [inputs.Shape(inputs.SHAPE_SPHERE, (21.0, 21.0, 21.0), 12.0)])
+b = api.Batch([plan], cell, [inputs.Shape(inputs.SHAPE_SPHERE, ({n} / 2,) * 3, 12.0)])
 b.forward()
 b.dl_dmean[0].fill_(1.0)
 b.backward()
@@ -46,18 +47,19 @@ assert torch.isfinite(b.dl_dcell[0]).all() and b.dl_dcell[0].abs().sum().item() 
 """)
 
 
-def test_batched_rows():
-    # 256 rows of 32: 48 KB of lines and row terms, and the stage table beside them
-    run("""
+# 256 rows of 32: 48 KB of lines and row terms, and the stage tables (1120 bytes) beside them; 273 of 28: 46.9 KB
+@pytest.mark.parametrize("n,rows", [(32, 256), (28, 273)])
+def test_batched_rows(n, rows):
+    run(f"""
 import torch
 from paper_2303_13435_gb300 import api, inputs
-plan = api.Plan(32, 0.05, inputs.linear_edges(inputs.nyquist_q(0.05), 20))
-plan.set_tiles(256, 0)
+plan = api.Plan({n}, 0.05, inputs.linear_edges(inputs.nyquist_q(0.05), 20))
+plan.set_tiles({rows}, 0)
 cell = torch.rand((6, 6, 6), device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
-shape = inputs.Shape(inputs.SHAPE_SPHERE, (16.0, 16.0, 16.0), 12.0)
+shape = inputs.Shape(inputs.SHAPE_SPHERE, ({n} / 2,) * 3, 12.0)
 b = api.Batch([plan], cell, [shape])
 bins = b.forward()[0]
-one = api.fft_intensity_tiled(api.Plan(32, 0.05, plan.edges), cell, shape)
+one = api.fft_intensity_tiled(api.Plan({n}, 0.05, plan.edges), cell, shape)
 ok = bins[api.BIN_COUNT] > 0
 assert torch.allclose(bins[api.BIN_MEAN][ok], one[api.BIN_MEAN][ok], rtol=1e-5)
 """)
