@@ -284,10 +284,7 @@ AdjRange ur_adj_range(const ur_plan* p, const ShapeArgs& sh, bool want_mask) {
 
 // columns with kx^2 + ky^2 at or beyond the closing threshold have zero scales at every kz: the
 // adjoint z pass leaves them unwritten and its y pass reads them as zeros
-int ur_k2_zero(const ur_plan* p) {
-  const int64_t t = p->thr_host[p->nbins];
-  return t < 0x7fffffff ? (int)t : 0x7fffffff;
-}
+int ur_k2_zero(const ur_plan* p) { return (int)p->thr_host[p->nbins]; }
 
 // Blocks of the generic row pass: as many cell rows per block as fill its RB rows
 void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy) {

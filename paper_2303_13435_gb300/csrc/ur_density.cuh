@@ -14,27 +14,9 @@ struct ShapeArgs {
   float rb2;  // rows (y, z) with fl(dy dy + dz dz) > rb2 have a zero mask at every x (infinity: unknown)
 };
 
-// Mask value at voxel (x, y, z): every product and sum rounded separately
-// (no contraction), in the order of the ur_build_density contract.
-__device__ __forceinline__ float mask_at(const ShapeArgs& sh, int x, int y, int z) {
-  if (sh.kind == UR_SHAPE_ALL) return 1.f;
-  const float dx = __fsub_rn((float)x, sh.cx);
-  const float dy = __fsub_rn((float)y, sh.cy);
-  const float dz = __fsub_rn((float)z, sh.cz);
-  if (sh.kind == UR_SHAPE_SPHERE) {
-    const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-    return d2 <= __fmul_rn(sh.s, sh.s) ? 1.f : 0.f;
-  }
-  float p[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-    p[a] = fabsf(__fadd_rn(__fadd_rn(__fmul_rn(sh.r[a], dx), __fmul_rn(sh.r[3 + a], dy)), __fmul_rn(sh.r[6 + a], dz)));
-  if (sh.kind == UR_SHAPE_CUBE) return (p[0] <= sh.s && p[1] <= sh.s && p[2] <= sh.s) ? 1.f : 0.f;
-  return __fadd_rn(__fadd_rn(p[0], p[1]), p[2]) <= sh.s ? 1.f : 0.f;  // octahedron
-}
-
 // Per-row part of the predicate: the y and z terms are fixed along a row, so
-// they are formed once (with the same roundings) and only the x term varies.
+// they are formed once and only the x term varies.  Every product and sum is rounded separately (no
+// contraction), in the order of the ur_build_density contract.
 struct RowMask {
   int kind;
   float s, s2;
@@ -63,7 +45,7 @@ struct RowMask {
   __device__ __forceinline__ bool sphere_empty() const {
     return kind == UR_SHAPE_SPHERE && __fadd_rn(dy2, dz2) > s2;
   }
-  // Signed coordinate of axis a at x, rounded as in mask_at; nondecreasing or nonincreasing in x,
+  // Signed coordinate of axis a at x, rounded as in at; nondecreasing or nonincreasing in x,
   // since rounding to nearest is monotone
   __device__ __forceinline__ float coord(int a, float dx) const {
     return __fadd_rn(__fadd_rn(__fmul_rn(r0[a], dx), ry[a]), rz[a]);

@@ -380,16 +380,9 @@ __global__ void __launch_bounds__((ColCfg<N, MODE>::THREADS), (ColCfg<N, MODE>::
     // every thread votes for its own column (columns past the end count as beyond); in the
     // forward the vote's barrier also publishes the range reset above
     const bool beyond = __syncthreads_and(!valid || c2 >= __ldg(a.thr + a.nbins));
-    if (beyond) {  // uniform over the block
-      // adjoint: the output columns are zero; unless the caller reads them as zeros
-      // without loading (k2_zero), write them
-      if (MODE == P2_Z_ADJ && valid && a.k2_zero == 0x7fffffff) {
-        const long long dbase = (long long)(col / H) * a.Ad + (col - (col / H) * H);
-#pragma unroll
-        for (int q = 0; q < E; ++q) a.dst[dbase + (long long)(j + q * T) * a.Sd] = make_float2(0.f, 0.f);
-      }
-      return;
-    }
+    // uniform over the block (adjoint: the output columns are zero, and the y pass takes them as zeros
+    // without loading them: k2_zero)
+    if (beyond) return;
   }
   if (MODE == P2_Z_ADJ && binning) {  // staged by the blocks that transform
     for (int i = threadIdx.x; i <= a.nbins; i += blockDim.x) thr[i] = __ldg(a.thr + i);
@@ -410,7 +403,7 @@ __global__ void __launch_bounds__((ColCfg<N, MODE>::THREADS), (ColCfg<N, MODE>::
       const int y = j + q * T;
       v[q] = (valid && !row_outside(a.sh, y, z)) ? __ldg(src + q * step) : make_float2(0.f, 0.f);
     }
-  } else if (YINV && a.k2_zero != 0x7fffffff) {
+  } else if (YINV) {
     // adjoint y pass: elements with kx^2 + ky^2 >= k2_zero are zero (the z pass left them
     // unwritten) and are not read
     const float2* src = a.src + (valid ? sbase + (long long)j * a.S : 0);

@@ -415,7 +415,7 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
       const int kx = (int)((uint32_t)c - o * dv.h.d);
       const bool valid = c < a.ncols;
       if (INV) {
-        s_ld[t] = !valid ? make_int2(0, N) : a.k2_zero == 0x7fffffff ? make_int2(0, 0) : beyond_range(kx, a.k2_zero, N);
+        s_ld[t] = !valid ? make_int2(0, N) : beyond_range(kx, a.k2_zero, N);
         if (a.row_skip) s_st[t] = valid ? row_range(a.sh, a.gen_z0 + (int)o, N) : make_int2(0, 0);
       } else {
         s_ld[t] = !valid ? make_int2(0, 0) : a.row_skip ? row_range(a.sh, a.gen_z0 + (int)o, N) : make_int2(0, N);
@@ -424,23 +424,14 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
   }
   if ((MODE == COL_ZBIN && a.nbins > 0 && !a.fout) || (MODE == COL_ZADJ && a.nbins > 0)) {
     // a tile whose columns all lie at or beyond the closing threshold reaches no bin: nothing to bin,
-    // or zero output (left unwritten when the y pass reads it as zeros, k2_zero)
+    // or zero output, which the y pass takes as zeros without loading it (k2_zero)
     bool beyond = true;
     for (int t = threadIdx.x; t < a.TX && c0 + t < a.ncols; t += blockDim.x) {
       const uint32_t o = dv.h.div((uint32_t)(c0 + t));
       const int kx = (int)((uint32_t)(c0 + t) - o * dv.h.d), ky = (int)o < a.M ? (int)o : (int)o - N;
       beyond = beyond && kx * kx + ky * ky >= __ldg(a.thr + a.nbins);
     }
-    if (__syncthreads_and(beyond)) {
-      if (MODE == COL_ZADJ && a.k2_zero == 0x7fffffff) {
-        const ColSt<MODE, INV> st(a, dv, c0, nullptr);
-        for (int f = threadIdx.x; f < a.TX * N; f += blockDim.x) {
-          const int i = (int)dv.tx.div((uint32_t)f);
-          st.first(f - i * a.TX, i, 1).put(make_float2(0.f, 0.f));
-        }
-      }
-      return;
-    }
+    if (__syncthreads_and(beyond)) return;
   }
   if (MODE != COL_Y && a.nbins > 0) {
     for (int j = threadIdx.x; j <= a.nbins; j += blockDim.x) thr[j] = __ldg(a.thr + j);
@@ -998,7 +989,6 @@ ColArgs ur_col_args(const ur_plan* p) {
   a.stw32 = p->stw + p->stw_32_off;
   a.thr = p->thr;
   a.lut = p->binlut;
-  a.k2_zero = 0x7fffffff;
   a.vs = p->vsinc;
   a.crs = p->bincoarse;
   a.crs_shift = p->coarse_shift;

@@ -52,8 +52,7 @@ struct ColArgs {
   int out_lo, out_cnt; // adjoint z pass: write only the planes z in [out_lo, out_lo + out_cnt), at
                        // z - out_lo (out_cnt = 0: every plane)
   int k2_zero;         // adjoint: spectrum columns with kx^2 + ky^2 >= k2_zero are zero; the z pass
-                       // may leave them unwritten and the y pass does not read them (0x7fffffff:
-                       // none)
+                       // may leave them unwritten and the y pass does not read them
 };
 
 // generic adjoint row pass (one block: up to RB rows wrapping onto G neighbouring cell rows)

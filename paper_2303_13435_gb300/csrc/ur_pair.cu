@@ -224,17 +224,9 @@ __global__ void __launch_bounds__(PairCfg<N, MODE>::THREADS, (PairCfg<N, MODE>::
   const unsigned dstep = (unsigned)(T * a.Sd * 8);
   if (skip_mode) {
     const bool beyond = __syncthreads_and(!valid || c2 >= __ldg(a.thr + nb));
-    if (beyond) {  // uniform over the block
-      // adjoint: the output columns are zero; unless the caller reads them as zeros without loading
-      // (k2_zero), write them
-      if (MODE == P2_Z_ADJ && valid && a.k2_zero == 0x7fffffff) {
-        const C2 zero = {0ull, 0ull};
-#pragma unroll
-        for (int q = 0; q < E; ++q)
-          c2_store(at_step(da + j * a.Sd, q, dstep), at_step(db + j * a.Sd, q, dstep), hasb, zero);
-      }
-      return;
-    }
+    // uniform over the block (adjoint: the output columns are zero, and the y pass takes them as zeros
+    // without loading them: k2_zero)
+    if (beyond) return;
   }
   if (MODE == P2_Z_ADJ && binning) {
     for (int i = threadIdx.x; i <= nb; i += Cfg::THREADS) thr[i] = __ldg(a.thr + i);
