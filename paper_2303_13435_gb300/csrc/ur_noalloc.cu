@@ -64,7 +64,7 @@ extern "C" ur_status ur_fft_intensity_noalloc(const ur_plan* p, const void* ed, 
   UR_REQUIRE(need <= (size_t)UR_NOALLOC_SCRATCH_BYTES,
              "ur_fft_intensity_noalloc: this plan needs %zu bytes of intermediate (nz * N * (N/2+1) * 8); the built-in "
              "scratch holds %zu bytes -- use ur_fft_intensity with a workspace",
-             need, (size_t)UR_NOALLOC_SCRATCH_BYTES);
+             (size_t)p->nz * p->n * p->H * sizeof(float2), (size_t)UR_NOALLOC_SCRATCH_BYTES);
   UR_REQUIRE(((uintptr_t)ed % 8) == 0, "ur_fft_intensity_noalloc: ed must be 8-byte aligned");
   UR_TRY(ur_fault_point("fft_intensity"));
   void* scratch = nullptr;
