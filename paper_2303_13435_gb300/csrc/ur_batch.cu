@@ -105,7 +105,7 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     }
     const size_t need = ur_workspace_size(p, bwd ? (UR_WS_FORWARD | UR_WS_BACKWARD) : UR_WS_FORWARD);
     UR_REQUIRE(it.ws_bytes >= need, "ur_batch_create: item %d workspace %zu < %zu bytes", i, it.ws_bytes, need);
-    const int n = p->n, H = p->H, M = p->M, nb = p->nbins;
+    const int n = p->n, H = p->H, nb = p->nbins;
     if (nb > maxnb) maxnb = nb;
     const double n3 = (double)n * n * n;
     float2* X = (float2*)it.ws;
@@ -131,7 +131,6 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     r.N = n;
     r.RB = p->row_rb;
     r.nst = p->sched_m.nst;
-    r.gen = 1;
     r.sched = p->d_sched + UR_MAX_STAGES;
     s_rows[i + 1] = s_rows[i] + (r.ra.nrows + r.RB - 1) / r.RB;
     r.ra.skip_empty = sh.rb2 < INFINITY && !weights;

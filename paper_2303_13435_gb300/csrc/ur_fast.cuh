@@ -54,7 +54,7 @@ struct GradArgs {
 // one item of a batched generic row pass
 struct BatchRowsItem {
   RowArgs ra;
-  int N, RB, nst, gen;
+  int N, RB, nst;
   const StageInfo* sched;
 };
 

@@ -60,7 +60,8 @@ struct NoSt {
 
 // GEN = 1: the row's density is generated here (Sec. 2.3 tile + mask) instead of read.
 // Body of one block (block index blk); shared by the single-plan and batched launches.
-template <int GEN, typename T>
+// IO: the first stage reads stored rows from global memory (nst >= 2).
+template <int GEN, typename T, bool IO = false>
 __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, const StageInfo* __restrict__ sched,
                                               int nst, long long blk) {
   extern __shared__ float2 smem[];
@@ -95,7 +96,7 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
     const bool any = __syncthreads_or(some);
     if (ra.skip_empty && !any) return;
   }
-  if (GEN == 0 && nst >= 2) {
+  if constexpr (IO) {
     // stored rows: the first stage reads them from global memory instead of from a copy in shared
     // memory (720^3 FP16 rows 1688 -> 1232 us; generated rows measured slower that way)
     auto stored = [&](int t, int m) -> float2 {
@@ -156,10 +157,10 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
   }
 }
 
-template <int GEN, typename T>
+template <int GEN, typename T, bool IO>
 __global__ void __launch_bounds__(256, 4) k_rows_r2c(RowArgs ra, int N, int RB, const StageInfo* __restrict__ sched,
                                                      int nst) {
-  rows_r2c_body<GEN, T>(ra, N, RB, sched, nst, blockIdx.x);
+  rows_r2c_body<GEN, T, IO>(ra, N, RB, sched, nst, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -919,10 +920,12 @@ ur_status ur_configure_kernels(ur_plan* p) {
   // the runtime-radix kernels accept any tile shape up to the per-block limit
   // (ur_plan_set_tiles may change it), so they get the largest dynamic size once
   const int kMaxDyn = 200 * 1024;
-  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
-  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, __half>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
-  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<1, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
-  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<2, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, __half, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<0, __half, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<1, float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
+  UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_r2c<2, float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
   UR_CUDA_CHECK(cudaFuncSetAttribute(k_cols<COL_Y, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
   UR_CUDA_CHECK(cudaFuncSetAttribute(k_cols<COL_Y, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
   UR_CUDA_CHECK(cudaFuncSetAttribute(k_cols<COL_ZBIN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
@@ -1024,11 +1027,19 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
     } else {
       const int grid_rows = (int)((r.nrows + p->row_rb - 1) / p->row_rb);
       const StageInfo* sm = p->d_sched + UR_MAX_STAGES;
-      if (gen == 2) k_rows_r2c<2, float><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, p->sched_m.nst);
-      else if (gen) k_rows_r2c<1, float><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, p->sched_m.nst);
-      else if (p->ed_dtype == UR_F32)
-        k_rows_r2c<0, float><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, p->sched_m.nst);
-      else k_rows_r2c<0, __half><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, p->sched_m.nst);
+      // stored rows that leave half of the SMs idle are short of time for one block, not of shared-memory
+      // bandwidth, and the first stage from global memory costs registers: 16^3 10.2 us against 6.3, 48^3
+      // 13.0 against 10.9; 90^3 (126 blocks) 13.8 against 14.1
+      const int nst = p->sched_m.nst;
+      const bool io = nst >= 2 && grid_rows >= p->num_sms / 2, f32 = p->ed_dtype == UR_F32;
+#define UR_ROWS(...) k_rows_r2c<__VA_ARGS__><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, nst)
+      if (gen == 2) UR_ROWS(2, float, false);
+      else if (gen) UR_ROWS(1, float, false);
+      else if (io && f32) UR_ROWS(0, float, true);
+      else if (io) UR_ROWS(0, __half, true);
+      else if (f32) UR_ROWS(0, float, false);
+      else UR_ROWS(0, __half, false);
+#undef UR_ROWS
       UR_LAUNCH_CHECK("k_rows_r2c");
     }
     ur_timing_end(s);
@@ -1250,8 +1261,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_rows(const BatchRowsItem* __re
                                                        const long long* __restrict__ start, int count) {
   const int i = batch_item(start, count, blockIdx.x);
   const BatchRowsItem& it = items[i];
-  if (it.gen) rows_r2c_body<1, float>(it.ra, it.N, it.RB, it.sched, it.nst, blockIdx.x - __ldg(start + i));
-  else rows_r2c_body<0, float>(it.ra, it.N, it.RB, it.sched, it.nst, blockIdx.x - __ldg(start + i));
+  rows_r2c_body<1, float>(it.ra, it.N, it.RB, it.sched, it.nst, blockIdx.x - __ldg(start + i));
 }
 
 template <int MODE, bool INV>
