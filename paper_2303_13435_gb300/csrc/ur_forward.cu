@@ -72,25 +72,23 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
   const int M = N >> 1, H = M + 1;
   const long long r0 = blk * RB;
   const FastDiv dm((uint32_t)M), dh((uint32_t)H);
-  // generated rows (r = p N + y < 2^31): what a row shares is formed once, by one thread per row
-  RowMask* rms = reinterpret_cast<RowMask*>(smem + (size_t)RB * M);
-  int* crow = reinterpret_cast<int*>(rms + RB);  // cell offset of the row; -1: past the last row
-  const FastDiv du((uint32_t)(GEN ? ra.ucell : 1));
+  // generated rows (r = p N + y < 2^31): what a row shares is formed once, by one thread per row.  Lattice
+  // samples (GEN = 2) form the mask's row terms anew: they are few against a sample's arithmetic, and the
+  // shared memory is worth more to its cell reads as L1.
+  RowMask* rms = reinterpret_cast<RowMask*>(smem + (size_t)RB * M);  // GEN = 1 (ur_row_smem)
+  int* crow = reinterpret_cast<int*>(rms + RB);                       // cell offset of the row
+  const FastDiv du((uint32_t)(GEN ? ra.ucell : 1)), dn((uint32_t)N);
   if (GEN) {
-    const FastDiv dn((uint32_t)N);
     bool some = false;
     for (int t = threadIdx.x; t < RB; t += blockDim.x) {
       const long long r = r0 + t;
-      if (r >= nrows) {
-        crow[t] = -1;
-        continue;
-      }
+      if (r >= nrows) break;
       const int p = (int)dn.div((uint32_t)r), y = (int)r - p * N, z = ra.z0 + p;
-      RowMask rm;
-      rm.init(ra.sh, y, z);
-      rms[t] = rm;
-      crow[t] = (int)(du.mod((uint32_t)(z + ra.oz)) * ra.ucell + du.mod((uint32_t)(y + ra.oy)));
-      some = some || !rm.empty(ra.sh);
+      if (GEN == 1) {
+        rms[t].init(ra.sh, y, z);
+        crow[t] = (int)(du.mod((uint32_t)(z + ra.oz)) * ra.ucell + du.mod((uint32_t)(y + ra.oy)));
+      }
+      some = some || !row_outside(ra.sh, y, z);
     }
     // rows outside the particle are not written when the y pass knows to skip them
     const bool any = __syncthreads_or(some);
@@ -113,22 +111,26 @@ __device__ __forceinline__ void rows_r2c_body(const RowArgs& ra, int N, int RB, 
       if (r < nrows) {
         if (GEN) {
           const int x = 2 * m, U = ra.ucell;
-          const int c0 = GEN == 2 ? 0 : (int)du.mod((uint32_t)(x + ra.ox));
-          const int c1 = c0 + 1 == U ? 0 : c0 + 1;
+          const int p = (int)dn.div((uint32_t)r), y = (int)r - p * N, z = ra.z0 + p;  // (GEN = 2)
           float m0, m1;
           if (ra.weights) {
             const float2 mw = __ldg(reinterpret_cast<const float2*>(ra.weights + ((long long)ra.z0 * N + r) * N + x));
             m0 = mw.x;
             m1 = mw.y;
+          } else if (GEN == 2) {
+            RowMask rm;
+            rm.init(ra.sh, y, z);
+            m0 = rm.at(x);
+            m1 = rm.at(x + 1);
           } else {
             m0 = rms[t].at(x);
             m1 = rms[t].at(x + 1);
           }
           if (GEN == 2) {
-            const int p = (int)(r / N), y = (int)(r - (long long)p * N), z = ra.z0 + p;
             v = make_float2(__fmul_rn(lattice_sample(ra.lat, ra.sh, ra.cell, U, x, y, z), m0),
                             __fmul_rn(lattice_sample(ra.lat, ra.sh, ra.cell, U, x + 1, y, z), m1));
           } else {
+            const int c0 = (int)du.mod((uint32_t)(x + ra.ox)), c1 = c0 + 1 == U ? 0 : c0 + 1;
             const float* cr = ra.cell + (long long)crow[t] * U;
             v = make_float2(__fmul_rn(__ldg(cr + c0), m0), __fmul_rn(__ldg(cr + c1), m1));
           }
@@ -1032,7 +1034,8 @@ static ur_status plane_pass(const ur_plan* p, RowArgs ra, int gen, long long npl
       // 13.0 against 10.9; 90^3 (126 blocks) 13.8 against 14.1
       const int nst = p->sched_m.nst;
       const bool io = nst >= 2 && grid_rows >= p->num_sms / 2, f32 = p->ed_dtype == UR_F32;
-#define UR_ROWS(...) k_rows_r2c<__VA_ARGS__><<<grid_rows, p->row_threads, p->row_smem, s>>>(r, n, p->row_rb, sm, nst)
+      const size_t smem = gen == 1 ? p->row_smem : (size_t)p->row_rb * p->M * sizeof(float2);
+#define UR_ROWS(...) k_rows_r2c<__VA_ARGS__><<<grid_rows, p->row_threads, smem, s>>>(r, n, p->row_rb, sm, nst)
       if (gen == 2) UR_ROWS(2, float, false);
       else if (gen) UR_ROWS(1, float, false);
       else if (io && f32) UR_ROWS(0, float, true);
