@@ -299,11 +299,11 @@ __global__ void __launch_bounds__(256) k_zoom_half(const __half* __restrict__ sr
   const int m = n_src / F, o = (n_out - m) / 2;
   const bool wide = n_out % 8 == 0 && ((uintptr_t)out % 16) == 0;  // rows start on 16-byte boundaries
   if (blockIdx.x >= (unsigned)(m * m)) {  // rows that no source row reaches
-    const long long r0 = (long long)(blockIdx.x - m * m) * UR_ZOOM_ZROWS;
-    for (long long r = r0; r < r0 + UR_ZOOM_ZROWS && r < (long long)n_out * n_out; ++r) {
-      const int Zr = (int)(r / n_out) - o, Yr = (int)(r % n_out) - o;
-      if (Zr >= 0 && Zr < m && Yr >= 0 && Yr < m) continue;
-      TO* row = out + r * n_out;
+    const unsigned r0 = (blockIdx.x - m * m) * UR_ZOOM_ZROWS;
+    int Z = (int)(r0 / (unsigned)n_out), Y = (int)(r0 - (unsigned)Z * n_out);
+    for (int i = 0; i < UR_ZOOM_ZROWS && Z < n_out; ++i, Z += Y + 1 == n_out, Y = Y + 1 == n_out ? 0 : Y + 1) {
+      if ((unsigned)(Z - o) < (unsigned)m && (unsigned)(Y - o) < (unsigned)m) continue;
+      TO* row = out + ((long long)Z * n_out + Y) * n_out;
       if (wide) {
         for (int X = threadIdx.x; X < n_out * (int)sizeof(TO) / 16; X += blockDim.x)
           reinterpret_cast<uint4*>(row)[X] = make_uint4(0u, 0u, 0u, 0u);
@@ -488,8 +488,11 @@ extern "C" ur_status ur_zoom_density(int32_t n_src, int32_t src_dtype, const voi
   } while (0)
   ur_timing_begin("zoom", s);
   // FP16 sources with the usual factors and rows of whole 16-byte groups: k_zoom_half; every other
-  // factor, edge, alignment and FP32 sources: k_zoom
-  const bool fast = src_dtype == UR_F16 && n_src % 8 == 0 && ((uintptr_t)src % 16) == 0;
+  // factor, edge, alignment and FP32 sources: k_zoom.  Halving short rows without a box around them
+  // leaves k_zoom_half too few loads in flight (48 -> 24 3.3 us against 2.9, 96 -> 48 5.5 against 5.1, but
+  // 128 -> 64 5.9 against 8.6, and 7.2 against 15.4 in a box of 128).
+  const bool fast = src_dtype == UR_F16 && n_src % 8 == 0 && ((uintptr_t)src % 16) == 0 &&
+                    (f > 2 || n_src >= 128 || n_out > m);
 #define UR_ZOOM_HALF(F)                                                                                   \
   do {                                                                                                    \
     const int threads = n_src / 8 >= 256 ? 256 : (n_src / 8 + 31) / 32 * 32;                              \
@@ -497,7 +500,8 @@ extern "C" ur_status ur_zoom_density(int32_t n_src, int32_t src_dtype, const voi
       UR_CUDA_CHECK(cudaFuncSetAttribute(k_zoom_half<F, __half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
       UR_CUDA_CHECK(cudaFuncSetAttribute(k_zoom_half<F, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  \
     }                                                                                                     \
-    const unsigned zgrid = (unsigned)((long long)m * m + ((long long)n_out * n_out + UR_ZOOM_ZROWS - 1) / UR_ZOOM_ZROWS); \
+    const unsigned zgrid = (unsigned)((long long)m * m +                                                  \
+                                      (n_out > m ? ((long long)n_out * n_out + UR_ZOOM_ZROWS - 1) / UR_ZOOM_ZROWS : 0));     \
     if (out_dtype == UR_F16)                                                                              \
       k_zoom_half<F, __half><<<zgrid, threads, smem, s>>>((const __half*)src, n_src, n_out, (__half*)out); \
     else k_zoom_half<F, float><<<zgrid, threads, smem, s>>>((const __half*)src, n_src, n_out, (float*)out); \

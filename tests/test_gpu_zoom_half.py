@@ -23,7 +23,7 @@ def halves(n, top, seed):
     return bits.view(np.float16)
 
 
-@pytest.mark.parametrize("f,n_src", [(2, 8), (2, 24), (2, 40), (4, 8), (4, 24), (4, 40), (8, 8), (8, 24), (8, 40),
+@pytest.mark.parametrize("f,n_src", [(2, 8), (2, 24), (2, 128), (2, 136), (4, 8), (4, 24), (4, 40), (8, 8), (8, 24), (8, 40),
                                      (16, 16), (16, 48), (16, 80)])
 @pytest.mark.parametrize("out_dtype", ["f16", "f32"])
 def test_block_sums_are_exact(f, n_src, out_dtype):
@@ -41,12 +41,12 @@ def test_block_sums_are_exact(f, n_src, out_dtype):
 @pytest.mark.parametrize("f", [2, 4, 8, 16])
 def test_values_that_are_not_finite(f):
     """As the sums of a source that does not start on a 16-byte boundary, which takes value by value."""
-    ed = halves(48, 0x5C00, f)
+    ed = halves(144, 0x5C00, f)
     ed[0, 1, 2], ed[20, 21, 47], ed[33, 0, 15], ed[33, 1, 14] = np.inf, -np.inf, np.nan, np.inf
     src = torch.from_numpy(ed).cuda()
-    flat = torch.empty(48 ** 3 + 1, dtype=torch.float16, device="cuda")
+    flat = torch.empty(144 ** 3 + 1, dtype=torch.float16, device="cuda")
     flat[1:] = src.flatten()
     for out_dtype in ("f16", "f32"):
-        got = [api.zoom_density(s, f, 48 // f, out_dtype=out_dtype).cpu().numpy().tobytes()
-               for s in (src, flat[1:].view(48, 48, 48))]
+        got = [api.zoom_density(s, f, 144 // f, out_dtype=out_dtype).cpu().numpy().tobytes()
+               for s in (src, flat[1:].view(144, 144, 144))]
         assert got[0] == got[1]
