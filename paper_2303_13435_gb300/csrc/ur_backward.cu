@@ -165,18 +165,27 @@ __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int
     __syncthreads();
     fft_lines<true, UR_EMAX>(buf, H, nrow, sched, nst, tw);
   }
-  // dL/dm = dL/drho * u
-  if (dl_dmask) {
+  // dL/dm = dL/drho * u.  Voxel weights are multiplied in here, where neighbouring threads read neighbouring
+  // ones, and not by the threads that sum a cell voxel's repeats
+  if (dl_dmask || weights) {
     const FastDiv dU((uint32_t)U);
     for (int f = threadIdx.x; f < nrow * M; f += blockDim.x) {
       const int t = (int)dM.div((uint32_t)f);
       const int m = f - t * M;
       const float2 zv = buf[t * H + m];
-      const int c0 = (int)dU.mod((uint32_t)(2 * m + ox)), c1 = c0 + 1 == U ? 0 : c0 + 1;
-      const float* crow = g.cell + ((long long)cz * U + cy0 + rows[t].g) * U;
-      *reinterpret_cast<float2*>(dl_dmask + ((long long)rows[t].z * N + rows[t].y) * N + 2 * m) =
-          make_float2(zv.x * inv_n3 * __ldg(crow + c0), zv.y * inv_n3 * __ldg(crow + c1));
+      const long long vox = ((long long)rows[t].z * N + rows[t].y) * N + 2 * m;
+      if (dl_dmask) {
+        const int c0 = (int)dU.mod((uint32_t)(2 * m + ox)), c1 = c0 + 1 == U ? 0 : c0 + 1;
+        const float* crow = g.cell + ((long long)cz * U + cy0 + rows[t].g) * U;
+        *reinterpret_cast<float2*>(dl_dmask + vox) =
+            make_float2(zv.x * inv_n3 * __ldg(crow + c0), zv.y * inv_n3 * __ldg(crow + c1));
+      }
+      if (weights) {
+        const float2 w = __ldg(reinterpret_cast<const float2*>(weights + vox));
+        buf[t * H + m] = make_float2(w.x != 0.f ? zv.x * inv_n3 * w.x : 0.f, w.y != 0.f ? zv.y * inv_n3 * w.y : 0.f);
+      }
     }
+    if (weights) __syncthreads();
   }
   // dL/du = sum of dL/drho * m over the repeats: task (cell row, share of its rows, cell column)
   const float* bufr = reinterpret_cast<const float*>(buf);
@@ -192,11 +201,7 @@ __device__ __forceinline__ void rows_grad_body(const GenGradArgs& g, int bx, int
       const RowMask& rm = rows[t].rm;
       const float* line = bufr + (size_t)t * 2 * H;
       if (weights) {
-        const float* w = weights + ((long long)rows[t].z * N + rows[t].y) * N;
-        for (int x = x0; x < N; x += U) {
-          const float m = __ldg(w + x);
-          if (m != 0.f) sum += line[x] * inv_n3 * m;
-        }
+        for (int x = x0; x < N; x += U) sum += line[x];
       } else {
         for (int x = x0; x < N; x += U) {
           const float m = rm.at(x);
