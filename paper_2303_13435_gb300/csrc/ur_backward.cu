@@ -291,8 +291,9 @@ AdjRange ur_adj_range(const ur_plan* p, const ShapeArgs& sh, bool want_mask) {
 // adjoint z pass leaves them unwritten and its y pass reads them as zeros
 int ur_k2_zero(const ur_plan* p) { return (int)p->thr_host[p->nbins]; }
 
-// Blocks of the generic row pass: as many cell rows per block as fill its RB rows
-void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy) {
+// Blocks of the generic row pass: as many cell rows per block as fill its RB rows, but not so many that a
+// small grid has fewer than `least` blocks
+void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int least, int* gx, long long* gy) {
   const int U = g->U;
   g->zlo = rg.zlo;
   g->zhi = rg.zhi;
@@ -311,6 +312,7 @@ void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy) 
   g->G = g->RB / per;
   if (g->G < 1) g->G = 1;
   if (g->G > U) g->G = U;
+  while (g->G > 1 && U * ((U + g->G - 1) / g->G) < least) g->G = (g->G + 1) / 2;
   *gx = (g->G * per + g->RB - 1) / g->RB;
   *gy = (long long)U * ((U + g->G - 1) / g->G);
 }
@@ -489,7 +491,7 @@ extern "C" ur_status ur_backward(const ur_plan* p, const double* dl_dmean, const
   ga.dl_dcell = dl_dcell;
   int gx = 0;
   long long gy = 0;
-  ur_grad_blocks(rg, &ga, &gx, &gy);
+  ur_grad_blocks(rg, &ga, p->num_sms, &gx, &gy);
   if (gy == 0) return UR_OK;
   const size_t smem = ur_grad_smem(p);
   UR_CUDA_CHECK(cudaFuncSetAttribute(k_rows_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -238,7 +238,7 @@ extern "C" ur_status ur_batch_create(int32_t count, const ur_batch_item* items, 
     g.g.dl_dmask = it.dl_dmask;
     g.g.dl_dcell = it.dl_dcell;
     long long gy = 0;
-    ur_grad_blocks(rg, &g.g, &g.gx, &gy);
+    ur_grad_blocks(rg, &g.g, p->num_sms / count, &g.gx, &gy);
     s_grad[i + 1] = s_grad[i] + (long long)g.gx * gy;
     smem_grad = std::max(smem_grad, ur_grad_smem(p));
   }

@@ -120,7 +120,7 @@ struct AdjRange {
 };
 AdjRange ur_adj_range(const ur_plan* p, const ShapeArgs& sh, bool want_mask);
 int ur_k2_zero(const ur_plan* p);
-void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int* gx, long long* gy);
+void ur_grad_blocks(const AdjRange& rg, GenGradArgs* g, int least, int* gx, long long* gy);
 size_t ur_grad_smem(const ur_plan* p);
 size_t ur_row_smem(int rb, int M);
 ColArgs ur_col_args(const ur_plan* p);
