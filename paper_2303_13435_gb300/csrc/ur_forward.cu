@@ -21,9 +21,11 @@
 
 #include "ur_fast.cuh"
 
-// Consecutive |kz| per thread in the binning and scaling walks; lanes read BIN_CHUNK values apart in
+// Consecutive |kz| per thread in the binning and scaling walks; lanes read that many values apart in
 // shared memory, so an odd number spreads them over the banks (8 -> 9: 378^3 z + bins 253 -> 245 us, adjoint
 // z 285 -> 268; 64 particles 3627 -> 3461 and 4374 -> 4059; 7 and 11 within 3 % of 9)
+// (Longer where a tile would take two rounds, shorter where tiles of short lines have fewer values per thread:
+// ur_col_args.)
 #define BIN_CHUNK 9
 
 // ---------------------------------------------------------------------------
@@ -302,14 +304,14 @@ __device__ __forceinline__ void store_columns(const ColArgs& a, const ColDivs& d
 }
 
 // Walk the (column, |kz|) pairs of the block's spectrum columns in chunks of
-// BIN_CHUNK consecutive |kz| = m.  k^2 = kx^2 + ky^2 + m^2 grows with m, so the
+// a.walk consecutive |kz| = m.  k^2 = kx^2 + ky^2 + m^2 grows with m, so the
 // bin index only moves forward inside a chunk.  kz = m and kz = N - m share k^2.
 // Op(t, m, bin, weight) is called for every pair.
 template <typename Op>
 __device__ __forceinline__ void walk_bins(const ColArgs& a, const ColDivs& dv, const int32_t* __restrict__ thr,
                                           long long c0, Op op) {
   const int M = a.M, H = a.H, N = a.N;
-  const int nch = (H + BIN_CHUNK - 1) / BIN_CHUNK;
+  const int len = a.walk, nch = (H + len - 1) / len;
   const int ntask = a.TX * nch;
   const FastDiv dch((uint32_t)nch);
   for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
@@ -322,8 +324,8 @@ __device__ __forceinline__ void walk_bins(const ColArgs& a, const ColDivs& dv, c
     const int ky = kyi < M ? kyi : kyi - N;
     const int c2 = kx * kx + ky * ky;
     const float w = (kx == 0 || kx == M) ? 1.f : 2.f;
-    const int m0 = ch * BIN_CHUNK;
-    const int m1 = min(m0 + BIN_CHUNK, M + 1);
+    const int m0 = ch * len;
+    const int m1 = min(m0 + len, M + 1);
     int cur = bin_search(thr, a.nbins, c2 + m0 * m0);
     // voxel-sinc factor of the column (kx, ky); the kz part is applied per element
     const float cs = a.vs ? __ldg(a.vs + kx) * __ldg(a.vs + (ky < 0 ? -ky : ky)) : 1.f;
@@ -425,17 +427,6 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
       }
     }
   }
-  if ((MODE == COL_ZBIN && a.nbins > 0 && !a.fout) || (MODE == COL_ZADJ && a.nbins > 0)) {
-    // a tile whose columns all lie at or beyond the closing threshold reaches no bin: nothing to bin,
-    // or zero output, which the y pass takes as zeros without loading it (k2_zero)
-    bool beyond = true;
-    for (int t = threadIdx.x; t < a.TX && c0 + t < a.ncols; t += blockDim.x) {
-      const uint32_t o = dv.h.div((uint32_t)(c0 + t));
-      const int kx = (int)((uint32_t)(c0 + t) - o * dv.h.d), ky = (int)o < a.M ? (int)o : (int)o - N;
-      beyond = beyond && kx * kx + ky * ky >= __ldg(a.thr + a.nbins);
-    }
-    if (__syncthreads_and(beyond)) return;
-  }
   if (MODE != COL_Y && a.nbins > 0) {
     for (int j = threadIdx.x; j <= a.nbins; j += blockDim.x) thr[j] = __ldg(a.thr + j);
     if (MODE == COL_ZBIN) {
@@ -447,7 +438,18 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, long long blk) {
       }
     }
   }
-  __syncthreads();
+  // a tile whose columns all lie at or beyond the closing threshold reaches no bin: nothing to bin, or zero
+  // output, which the y pass takes as zeros without loading it (k2_zero).  The vote is also the barrier
+  // that publishes the tables.
+  bool beyond = a.nbins > 0 && (MODE == COL_ZADJ || (MODE == COL_ZBIN && !a.fout));
+  if (beyond) {
+    for (int t = threadIdx.x; t < a.TX && c0 + t < a.ncols; t += blockDim.x) {
+      const uint32_t o = dv.h.div((uint32_t)(c0 + t));
+      const int kx = (int)((uint32_t)(c0 + t) - o * dv.h.d), ky = (int)o < a.M ? (int)o : (int)o - N;
+      beyond = beyond && kx * kx + ky * ky >= __ldg(a.thr + a.nbins);
+    }
+  }
+  if (__syncthreads_and(beyond)) return;
   if (MODE == COL_ZBIN && a.nbins > 0) {
     // bins this tile can reach: k^2 in [min kx^2+ky^2, max kx^2+ky^2 + (N/2)^2]
     if (threadIdx.x < a.TX && c0 + threadIdx.x < a.ncols) {
@@ -998,6 +1000,9 @@ ColArgs ur_col_args(const ur_plan* p) {
   a.crs = p->bincoarse;
   a.crs_shift = p->coarse_shift;
   a.nbins = p->nbins;
+  // a tile's walks in one round of the block's threads
+  a.walk = p->n < 64 ? 1 : BIN_CHUNK;
+  while (a.walk < 15 && a.TX * ((a.H + a.walk - 1) / a.walk) > p->col_threads) a.walk += 2;
   return a;
 }
 

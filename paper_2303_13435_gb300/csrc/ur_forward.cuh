@@ -51,6 +51,7 @@ struct ColArgs {
   ShapeArgs sh;        // y pass, nobody reads them and they are not written
   int out_lo, out_cnt; // adjoint z pass: write only the planes z in [out_lo, out_lo + out_cnt), at
                        // z - out_lo (out_cnt = 0: every plane)
+  int walk;            // runtime-radix z passes: consecutive |kz| per thread of a walk over the bins (odd)
   int k2_zero;         // adjoint: spectrum columns with kx^2 + ky^2 >= k2_zero are zero; the z pass
                        // may leave them unwritten and the y pass does not read them
 };
