@@ -152,7 +152,10 @@ __device__ __forceinline__ float2 ld_pair<__half>(const __half* p) {
 // Values per thread: 8, and 16 for stored rows of N = 1024, where a row then is one warp as it is below
 // (warp barriers only): 1024^3 FP16 rows 2270 -> 1849 us, FP16 slabs of the streamed forward 302 -> 174 us.
 // Generated rows (541 -> 597 us) and the adjoint rows (2612 -> 3056 us) at 1024, with 64 and 80 registers,
-// and two and more warps per row (2048 on: 1-3 %) were slower with 16.
+// and rows of 2048 (1-3 %) were slower with 16 while the stage tables held rows of E entries per k.  With the
+// present tables 16 is faster there too (1024: generated 452 -> 406, adjoint 2182 -> 1867 us; 2048: generated
+// 2685 -> 2230, stored FP16 15670 -> 12405, adjoint 18884 -> 15433), for transforms of radices 16, 16, 2 whose
+// rounding error is larger than that of 8, 8, 8 (1.00e-7 against 0.98e-7): not taken yet.
 template <int N, int GEN>
 struct RowCfg {
   static constexpr int E = GEN == 0 ? UR_FAST_STORED_ROW_E(N) : 8;
@@ -309,10 +312,12 @@ __global__ void __launch_bounds__((RowCfg<N, GEN>::THREADS), (RowCfg<N, GEN>::E 
 // Columns.  Block = TX columns x L/E threads; thread (j, c), c fastest, so a
 // warp reads whole row segments of TX consecutive columns.
 // ---------------------------------------------------------------------------
-// Values per thread and threads per block.  At 1024 the passes without binning hold 32 values per thread
-// (1024 = 32 32: one shared-memory exchange instead of two; 128 registers, two blocks of 256 threads): y 823 ->
-// 719 us, adjoint z 2540 -> 2475, adjoint y 1955 -> 1691; the binned pass keeps 16 (2200 -> 2461 us with 32: a
-// walk twice as long per thread).  512 points gain nothing by it (91 -> 113 us against pairs).  16 values per
+// Values per thread and threads per block.  At 1024 the adjoint's y pass holds 32 values per thread (1024 = 32 32:
+// one shared-memory exchange instead of two; 128 registers, two blocks of 256 threads): 2026 -> 1730 us.  The
+// forward y pass (850 -> 723) and the adjoint z pass (2489 -> 2467) would gain too, but with 32 there the
+// gradients of a fit are less accurate (cell gradient of a 1024^3 step against float64 5.4e-7 -> 6.9e-7: 17 and 8 %,
+// none by the adjoint's y pass), so they keep 16; the binned pass is slower with 32 (2154 -> 2475 us, of a full grid
+// 2305 -> 2612: a walk twice as long per thread).  512 points gain nothing by it (91 -> 113 us against pairs).  16 values per
 // thread take 64 registers and blocks of 512 threads, or 1024 for N >= 2048 so that a block still spans
 // at least two columns (16-byte row segments) of the half spectrum.
 template <int N, int MODE>

@@ -6,8 +6,8 @@
 
 // Values per column and thread of the column transforms: 8 up to 512 (pairs of columns, ur_pair.cu), 16
 // from 1024 on (single columns, ur_fast.cu: three radix-16 stages at 4096 instead of four radix-8
-// ones; measured 22-23 % faster steps), 32 at 1024 where nothing is binned (ColCfg)
-#define UR_FAST_COL_E(n, mode) ((n) == 1024 && (mode) != P2_Z_BIN ? 32 : 16)
+// ones; measured 22-23 % faster steps), 32 in the adjoint's y pass at 1024 (ColCfg)
+#define UR_FAST_COL_E(n, mode) ((n) == 1024 && ((mode) == P2_Y_INV || (mode) == P2_Y_INV_ROWS) ? 32 : 16)
 // ... and of the transforms of stored rows of n reals (generated rows and the adjoint rows: 8)
 #define UR_FAST_STORED_ROW_E(n) ((n) == 1024 ? 16 : 8)
 

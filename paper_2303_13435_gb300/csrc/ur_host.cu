@@ -463,7 +463,7 @@ extern "C" ur_status ur_plan_create(const ur_grid_desc* g, const double* edges, 
     // tables, one after the other: columns (N points; pairs, or 16 values per thread), rows (N/2 points)
     // with 8, stored rows where they take more, columns with 32
     const bool pair = ur_pair_supported(n);
-    const int erow = UR_FAST_STORED_ROW_E(n), e32 = UR_FAST_COL_E(n, P2_Y_FWD);
+    const int erow = UR_FAST_STORED_ROW_E(n), e32 = UR_FAST_COL_E(n, P2_Y_INV);
     const size_t cn = pair ? 2 * ur_pair_twiddles(n, nullptr) : ur_stage_twiddles(lg, 16, nullptr);
     const size_t cm = ur_stage_twiddles(lg - 1, 8, nullptr), cs = erow == 8 ? 0 : ur_stage_twiddles(lg - 1, erow, nullptr);
     const size_t c32 = e32 == 32 ? ur_stage_twiddles(lg, 32, nullptr) : 0;

@@ -18,9 +18,10 @@
 // 16-byte load is a packed operand and neighbouring lanes read neighbouring words.
 //
 // Measured against one column per group, us: z + bins of a 256^3 forward 62 -> 49; 512^3 step: y 106 -> 90, z + bins 258 -> 240, adjoint z 322 -> 276, adjoint y 220 -> 203.  The
-// shared-memory and L1 data pipe is now the busiest unit (65-68 %).  At 1024 pairs were slower
-// (y 932 -> 985, adjoint z 2538 -> 2684; z + bins of a full grid 2231 -> 2510 us: rows ky and -ky of a
-// plane lie in different 2 MB pages), so from 1024 on the columns are transformed one by one
+// shared-memory and L1 data pipe is now the busiest unit (65-68 %).  At 1024 pairs are slower than
+// single columns with 16 and 32 values per thread (y 723 -> 1362, z + bins 2154 -> 2890, of a full grid 2305 ->
+// 4114, adjoint z 2469 -> 3382, adjoint y 1730 -> 1986 us: row segments of 16 and 32 bytes, and rows ky and -ky
+// of a plane lie in different 2 MB pages), so from 1024 on the columns are transformed one by one
 // (ur_fast.cu).
 #include <vector>
 
